@@ -129,7 +129,8 @@ typedef struct {
 
 /* ---- run options ---------------------------------------------------------------------- */
 #define RTLFS_SCHED_PLAIN      0   /* queue in fault-list order, no heavy pre-assignment */
-#define RTLFS_SCHED_HEURISTIC  1   /* order by static cone size x toggle rate */
+#define RTLFS_SCHED_HEURISTIC  1   /* order by static cone size x toggle rate; the packed form (see
+                                      heavy_form) takes the list order unless heavy_frac > 0 */
 #define RTLFS_SCHED_MLP        2   /* order by the load predictor (falls back to heuristic
                                       when no weights are loaded) */
 
@@ -160,8 +161,13 @@ typedef struct {
                                 (made by a stopped run or rtlfs_checkpoint_load); the other
                                 options must match the stopped run's window, no_drop and
                                 light_cap (RTLFS_E_ARG otherwise) */
-    int32_t  heavy_form;     /* heavy kernel's record of differing nets: 0 = auto (the
-                                exact one unless it costs resident CTAs), 1 = a shared-memory
+    int32_t  heavy_form;     /* 0 = auto: the packed form (several faults per warp, in tiers of 1, 8,
+                                32 and 256 lanes per fault; windows of 64 cycles inside the ones
+                                asked for; light and heavy options then only decide which faults
+                                the counters call light or heavy) for designs of at most 4095
+                                levels and 2^27 nets, else as 1 unless its bitmap costs resident
+                                CTAs. Otherwise the light and heavy kernels with this record of
+                                differing nets: 1 = a shared-memory
                                 bit per net, 2 = a small shared filter plus cycle stamps on
                                 the values in global scratch (for designs whose per-net
                                 bitmap would crowd shared memory), 3 = as 2 with the
@@ -198,15 +204,17 @@ typedef struct {
     double   good_ms;        /* good-machine trace (all designs) */
     double   prep_ms;        /* features, predictor, queue order */
     double   faulty_ms;      /* light + heavy faulty-machine kernels */
-    double   light_ms;       /* light kernel alone */
-    double   heavy_ms;       /* promoted-fault heavy pass alone */
+    double   light_ms;       /* light kernel alone, or the packed form's first tier */
+    double   heavy_ms;       /* promoted-fault heavy pass alone, or the packed form's other tiers,
+                                each one's own time summed (they overlap) */
     uint64_t fault_cycles;   /* W = sum over faults of (cycle+1 if detected else T) */
     uint64_t node_evals;     /* sum of the per-fault propagation loads */
     uint64_t promoted;       /* light faults promoted to the heavy kernel */
     uint64_t heavy_initial;  /* faults assigned to the heavy kernel from cycle 0 */
     uint32_t n_launches;     /* kernels launched by the run */
     uint32_t heavy_form;     /* heavy kernel's record of differing nets in the run: 1 exact,
-                                2 stamped, 3 stamped with the node bitmap in global scratch */
+                                2 stamped, 3 stamped with the node bitmap in global scratch,
+                                4 the packed form */
     uint64_t light_evals;         /* node evaluations done by the light kernel */
     uint64_t light_fault_cycles;  /* fault-cycles completed by the light kernel */
     uint64_t heavy_evals;         /* node evaluations done by the heavy kernel */

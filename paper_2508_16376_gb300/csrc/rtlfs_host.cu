@@ -64,15 +64,15 @@ struct Design {
     std::vector<uint32_t> lvl_start;
     std::vector<uint16_t> node_level;
     std::vector<uint8_t> net_w;
-    std::vector<uint32_t> fo_off, fo_idx, dreg_off, dreg_idx, dreg_rec, reg_d, outport, out_net;
-    std::vector<uint4> netinfo;
+    std::vector<uint32_t> fo_off, fo_idx, fo_edge, dreg_off, dreg_idx, dreg_rec, reg_d, outport, out_net;
+    std::vector<uint4> netinfo, rec;
     std::vector<uint2> chunks;
     std::vector<float> cone;          // static fan-out cone size estimate per net (log2 scale)
     std::vector<float> net_static;    // [n_net][4] cone, level, register depth, width (scaled)
     DBuf<float> d_net_static;
-    DBuf<uint4> d_desc, d_netinfo;
+    DBuf<uint4> d_desc, d_netinfo, d_rec;
     DBuf<uint2> d_chunks;
-    DBuf<uint32_t> d_lvl_start, d_fo_off, d_fo_idx, d_dreg_off, d_dreg_idx, d_dreg_rec, d_reg_d,
+    DBuf<uint32_t> d_lvl_start, d_fo_off, d_fo_idx, d_fo_edge, d_dreg_off, d_dreg_idx, d_dreg_rec, d_reg_d,
         d_outport, d_out_net;
     DBuf<uint16_t> d_node_level, d_fo_lvl;
     std::vector<uint16_t> fo_lvl;
@@ -106,6 +106,9 @@ struct GoodLaunch {
     size_t smem_cl[5] = {};       // shared memory per CTA of each cluster launch
 };
 
+// Kernels of a window that are timed: light and heavy, or the packed tiers and the heavy kernel.
+constexpr size_t WIN_TIMED = PACK_TIERS + 1;
+
 struct rtlfs_ctx {
     int device = 0;
     GoodLaunch gl;
@@ -128,13 +131,27 @@ struct rtlfs_ctx {
     DBuf<unsigned long long> w_cnt64;
     DBuf<uint64_t> d_act;              // activation bitplane [F][ceil(Tmax/64)]
     DBuf<HeavyCarry> w_carry0, w_carry1;
+    // packed form: faults handed from tier to tier with their register diffs, the heavier
+    // tiers' survivors, and which faults count as heavy
+    DBuf<PackItem> pk_items[PACK_TIERS];
+    DBuf<uint32_t> pk_prom_r;
+    DBuf<uint64_t> pk_prom_v;
+    DBuf<HeavyCarry> pk_carry[PACK_TIERS - 2][2];   // [third tier on][window parity]
+    DBuf<uint32_t> pk_pool_r[PACK_TIERS - 2][2];
+    DBuf<uint64_t> pk_pool_v[PACK_TIERS - 2][2];
+    DBuf<uint32_t> pk_last_r;          // register diffs the last tier hands on in a window
+    DBuf<uint64_t> pk_last_v;
+    DBuf<uint8_t> pk_cls;
+    uint64_t pk_prom_cap = 0;
+    cudaStream_t s_tier[PACK_TIERS - 2] = {};   // third tier on (the last with the heavy kernel)
+    cudaEvent_t ev_pk[PACK_TIERS] = {};
     uint64_t w_pool_cap = 0;
     cudaEvent_t ev_wg = nullptr, ev_wl = nullptr;
     // the good-trace launch lists of one span of cycles run side by side: the first on the
     // caller's stream, the others on these, joined back through the events
     cudaStream_t s_gaux[5] = {};
     cudaEvent_t ev_gfork = nullptr, ev_gjoin[5] = {};
-    std::vector<cudaEvent_t> ev_win;   // [4][nw]: light start/end, heavy start/end
+    std::vector<cudaEvent_t> ev_win;   // [2 * WIN_TIMED][nw]: start/end of each kernel of a window
     cudaEvent_t ev[8] = {};
     DBuf<DevDesign> d_designs;
     DBuf<uint32_t> d_list_smem, d_list_glob, d_list_cl[5];
@@ -403,6 +420,51 @@ int build_design(rtlfs_ctx *ctx, Design &D, const rtlfs_node *nodes, uint32_t N,
         D.netinfo[e] = make_uint4(D.fo_off[e], D.fo_off[e + 1], D.dreg_off[e],
                                   (std::min<uint32_t>(nr, 255u) << 24) | port);
     }
+    // Everything the packed kernel reads of a net, in one 128-byte record.
+    D.fo_edge.resize(D.n_fo);
+    for (uint32_t e = 0; e < n_net; ++e)
+        for (uint32_t k = D.fo_off[e]; k < D.fo_off[e + 1]; ++k) {
+            const uint4 d = D.desc[D.fo_idx[k]];
+            const bool mux = meta_op(d.w) == OP_MUX2;
+            const int no = n_ops(meta_op(d.w));
+            uint32_t b = 0;
+            if (mux) b = (d.y == e ? 1u : 0u) | (d.z == e ? 2u : 0u) | (d.x == e ? 4u : 0u);
+            else b = (d.x == e ? 1u : 0u) | (no >= 2 && d.y == e ? 2u : 0u);
+            D.fo_edge[k] = (IR + D.fo_idx[k]) | b << 27;   // read only below 2^27 nets
+        }
+    D.rec.assign((size_t)n_net * 8, make_uint4(0, 0, 0, 0));
+    for (uint32_t e = 0; e < n_net; ++e) {
+        uint4 *r = &D.rec[(size_t)e * 8];
+        uint32_t c[8] = {}, l[8] = {};
+        for (uint32_t k = 0; k < 8 && D.fo_off[e] + k < D.fo_off[e + 1]; ++k) {
+            c[k] = D.fo_edge[D.fo_off[e] + k];
+            l[k] = (uint32_t)(uint16_t)(D.fo_lvl[D.fo_off[e] + k] << 4);
+        }
+        if (e >= IR) r[0] = D.desc[e - IR];
+        if (e >= IR && meta_op(r[0].w) == OP_MUX2) r[0] = make_uint4(r[0].y, r[0].z, r[0].x, r[0].w);
+        if (e >= IR) {
+            const int no = n_ops(meta_op(r[0].w));
+            r[0].w |= (no >= 3 ? 7u : no == 2 ? 3u : no == 1 ? 1u : 0u) << 4;
+            switch (meta_op(r[0].w)) {
+            case OP_AND: r[0].w |= PM_A; break;
+            case OP_OR: r[0].w |= PM_A | PM_B | PM_C; break;
+            case OP_XOR: r[0].w |= PM_B | PM_C; break;
+            case OP_NOT: r[0].w |= PM_B | PM_D; break;
+            case OP_ADD: case OP_SUB: r[0].w |= PM_SUM; break;
+            case OP_EQ: case OP_LT: r[0].w |= PM_CMP; break;
+            case OP_MUX2: r[0].w |= PM_C; break;
+            case OP_SHL: r[0].w |= PM_B | PM_LEFT; break;
+            case OP_CONCAT: r[0].w |= PM_B | PM_C | PM_LEFT; break;
+            case OP_SHR: case OP_SLICE: r[0].w |= PM_B; break;
+            default: break;
+            }
+        }
+        r[1] = D.netinfo[e];
+        if (ni_nreg(r[1].w) == 1) r[1].z = D.dreg_rec[D.dreg_off[e]];
+        r[2] = make_uint4(c[0], c[1], c[2], c[3]);
+        r[3] = make_uint4(c[4], c[5], c[6], c[7]);
+        r[4] = make_uint4(l[0] | l[1] << 16, l[2] | l[3] << 16, l[4] | l[5] << 16, l[6] | l[7] << 16);
+    }
     D.chunks.clear();
     for (uint32_t l = 0; l < NL; ++l) {
         for (uint32_t lo = D.lvl_start[l]; lo < D.lvl_start[l + 1]; lo += GOOD_BLOCK) {
@@ -464,6 +526,8 @@ int build_design(rtlfs_ctx *ctx, Design &D, const rtlfs_node *nodes, uint32_t N,
 int upload_design(rtlfs_ctx *ctx, Design &D) {
     CU(D.d_desc.upload(D.desc));
     CU(D.d_netinfo.upload(D.netinfo));
+    CU(D.d_fo_edge.upload(D.fo_edge));
+    CU(D.d_rec.upload(D.rec));
     CU(D.d_net_static.upload(D.net_static));
     CU(D.d_chunks.upload(D.chunks));
     CU(D.d_lvl_start.upload(D.lvl_start));
@@ -488,7 +552,7 @@ DevDesign dev_view(const Design &D) {
     v.n_chunks = (uint32_t)D.chunks.size();
     v.netinfo = D.d_netinfo.p; v.chunks = D.d_chunks.p;
     v.desc = D.d_desc.p; v.lvl_start = D.d_lvl_start.p; v.node_level = D.d_node_level.p;
-    v.net_w = D.d_net_w.p; v.fo_off = D.d_fo_off.p; v.fo_idx = D.d_fo_idx.p; v.fo_lvl = D.d_fo_lvl.p;
+    v.net_w = D.d_net_w.p; v.fo_off = D.d_fo_off.p; v.fo_idx = D.d_fo_idx.p; v.fo_lvl = D.d_fo_lvl.p; v.rec = D.d_rec.p; v.fo_edge = D.d_fo_edge.p;
     v.dreg_off = D.d_dreg_off.p; v.dreg_idx = D.d_dreg_idx.p; v.dreg_rec = D.d_dreg_rec.p; v.reg_d = D.d_reg_d.p;
     v.outport = D.d_outport.p; v.out_net = D.d_out_net.p; v.stim = D.d_stim.p;
     v.rows = D.d_rows.p; v.gcol = D.d_gcol.p;
@@ -851,6 +915,48 @@ HeavyScratch heavy_view(rtlfs_ctx *ctx) {
     return s;
 }
 
+// The packed faulty-machine form for the loaded designs.
+struct PackPlan {
+    bool use = false, multi = false;
+    int grid = 0;
+    int warps[PACK_TIERS] = {};
+    uint32_t evals[PACK_TIERS] = {};   // evaluations in a cycle beyond which a fault moves on
+};
+
+// The packed form runs whenever its tags can name the levels of every design and 27 bits its
+// nets. A run that names a heavy form asks for the light and heavy kernels.
+PackPlan plan_pack(rtlfs_ctx *ctx, int heavy_form) {
+    PackPlan p;
+    uint32_t nl = 1, mn = 1;
+    for (Design *D : ctx->designs) { nl = std::max(nl, D->n_levels); mn = std::max(mn, D->n_net); }
+    if (heavy_form != 0 || nl > PACK_LEVELS || mn > PACK_NETS) return p;
+    p.multi = ctx->designs.size() > 1;
+    p.grid = ctx->n_sm;
+    // With few faults the rounds of the slowest ones set the pace: faults move to a tier with
+    // more lanes early. With many the issue slots do: they move only when their cones outgrow
+    // what a tier handles in a few rounds, and the tiers' shares of an SM follow their work.
+    // (medium campaign, 658 faults per SM, windows of 128: 922 against 1402 ms; transient list,
+    // 197 per SM, windows of 256: 199 against 182)
+    const bool many = ctx->F > 400u * (uint32_t)ctx->n_sm;
+    const int w[2][PACK_TIERS] = {{5, 4, 4, 1}, {3, 5, 7, 1}};
+    const uint32_t e[2][PACK_TIERS] = {{6, 48, 160, 0xFFFFFFFFu}, {8, 64, 0xFFFFFFFFu, 0xFFFFFFFFu}};
+    for (int k = 0; k < PACK_TIERS; ++k) { p.warps[k] = w[many][k]; p.evals[k] = e[many][k]; }
+    p.use = true;
+    return p;
+}
+
+// Cycles per window of the packed form. Its kernels hand faults from tier to tier once a
+// window and the tiers of a window overlap those of the next, so the shortest window the
+// activation bitplane allows (64 cycles) is the fastest as long as the launches stay few:
+// `asked` (0: none) when 64 does not divide it, else 64, longer beyond 512 windows. (Windows of
+// 64 / 128 / 256: recorded loads 84 / 89 / 102 ms, no-drop 129 / 133 / 142, large 91 / 97 / 115.)
+uint32_t pack_window(uint32_t asked, uint32_t Tmax) {
+    if (asked % 64 != 0) return asked;
+    uint32_t w = 64;
+    while ((Tmax + w - 1) / w > 512 && (asked == 0 || (w < asked && asked % (2 * w) == 0))) w *= 2;
+    return w;
+}
+
 int ensure_sched_buffers(rtlfs_ctx *ctx) {
     std::vector<const float *> ptrs;
     for (Design *D : ctx->designs) ptrs.push_back(D->d_net_static.p);
@@ -953,12 +1059,13 @@ int checkpoint_matches(rtlfs_ctx *ctx, const rtlfs_ctx::Checkpoint &c, uint32_t 
 
 // Copy the campaign state after window w_end - 1 to the host (after the stream has drained).
 // pending[f] marks the faults still alive at the stop.
-int take_checkpoint(rtlfs_ctx *ctx, uint32_t nw, uint32_t w_end, uint32_t W, bool nodrop, int lcap,
+// The launches ran windows of W cycles; the checkpoint counts the caller's windows of WU.
+int take_checkpoint(rtlfs_ctx *ctx, uint32_t nw, uint32_t w_end, uint32_t W, uint32_t WU, bool nodrop, int lcap, bool packed,
                     std::vector<uint8_t> *pending) {
     rtlfs_ctx::Checkpoint &c = ctx->ck;
     const uint32_t F = ctx->F, wl = w_end - 1;
     c = rtlfs_ctx::Checkpoint{};
-    c.window = w_end; c.W = W; c.F = F; c.nodrop = nodrop ? 1u : 0u; c.lcap = (uint32_t)lcap;
+    c.window = w_end * W / WU; c.W = WU; c.F = F; c.nodrop = nodrop ? 1u : 0u; c.lcap = (uint32_t)lcap;
     for (Design *D : ctx->designs) { c.T.push_back(D->T); c.n_net.push_back(D->n_net); }
     uint32_t n_live = 0, n_carry = 0;
     unsigned long long pool_top = 0;
@@ -990,6 +1097,52 @@ int take_checkpoint(rtlfs_ctx *ctx, uint32_t nw, uint32_t w_end, uint32_t W, boo
         if (cyc <= D->T && D->n_net)
             CU(cudaMemcpy(row.data(), D->d_rows.p + (size_t)(cyc - 1) * D->n_net, (size_t)D->n_net * 8, cudaMemcpyDeviceToHost));
         c.rows.insert(c.rows.end(), row.begin(), row.end());
+    }
+    if (packed) {
+        // the heavier tiers' survivors join the carried ones
+        const uint32_t *pk32 = ctx->w_cnt32.p + 3 * (size_t)nw + 4;
+        const unsigned long long *pk64 = ctx->w_cnt64.p + 3 * (size_t)nw + 1;
+        for (int k = 0; k < PACK_TIERS - 2; ++k) {
+            uint32_t n = 0;
+            unsigned long long top = 0;
+            CU(cudaMemcpy(&n, pk32 + (PACK_TIERS - 1 + k) * (size_t)nw + wl, 4, cudaMemcpyDeviceToHost));
+            CU(cudaMemcpy(&top, pk64 + k * (size_t)nw + wl, 8, cudaMemcpyDeviceToHost));
+            if (n > F || top > ctx->w_pool_cap) return fail(ctx, RTLFS_E_CUDA, "inconsistent campaign counters");
+            std::vector<HeavyCarry> cv;
+            std::vector<uint32_t> pr;
+            std::vector<uint64_t> pv;
+            if ((r = get(cv, ctx->pk_carry[k][wl & 1].p, n)) || (r = get(pr, ctx->pk_pool_r[k][wl & 1].p, top)) ||
+                (r = get(pv, ctx->pk_pool_v[k][wl & 1].p, top)))
+                return r;
+            for (HeavyCarry &x : cv) { x.off += c.pool_r.size(); c.carry.push_back(x); }
+            c.pool_r.insert(c.pool_r.end(), pr.begin(), pr.end());
+            c.pool_v.insert(c.pool_v.end(), pv.begin(), pv.end());
+        }
+        // sorted as the light and heavy kernels leave them: light faults (at most the light
+        // capacity's register diffs) with their state in st_*, heavy ones in the pool
+        std::vector<uint8_t> cls;
+        if ((r = get(cls, ctx->pk_cls.p, F))) return r;
+        std::vector<uint32_t> light;
+        std::vector<HeavyCarry> heavy;
+        for (const HeavyCarry &x : c.carry) {
+            if (cls[x.fault]) { heavy.push_back(x); continue; }
+            light.push_back(x.fault);
+            c.st_nreg[x.fault] = (uint8_t)x.nreg;
+            for (uint32_t k = 0; k < x.nreg && k < (uint32_t)LIGHT_KR; ++k) {
+                c.st_r[(size_t)k * F + x.fault] = c.pool_r[x.off + k];
+                c.st_v[(size_t)k * F + x.fault] = c.pool_v[x.off + k];
+            }
+        }
+        for (uint32_t x : c.live) {
+            if (!cls[x]) { light.push_back(x); continue; }
+            heavy.push_back(HeavyCarry{x, c.st_nreg[x], c.pool_r.size()});
+            for (uint32_t k = 0; k < c.st_nreg[x]; ++k) {
+                c.pool_r.push_back(c.st_r[(size_t)k * F + x]);
+                c.pool_v.push_back(c.st_v[(size_t)k * F + x]);
+            }
+        }
+        c.live.swap(light);
+        c.carry.swap(heavy);
     }
     pending->assign(F, 0);
     for (uint32_t f : c.live) if (f < F) (*pending)[f] = 1;
@@ -1027,7 +1180,7 @@ int restore_checkpoint(rtlfs_ctx *ctx, uint32_t nw, uint32_t w_begin, uint32_t *
     CU(cudaMemcpyAsync(ctx->w_cnt32.p + 2 * (size_t)nw + wp, cnt + 1, 4, cudaMemcpyHostToDevice, s));
     CU(cudaMemsetAsync(ctx->w_cnt32.p + nw + wp, 0, 4, s));
     CU(cudaMemsetAsync(prom_total, 0, 4, s));
-    const uint32_t cyc = w_begin * c.W;
+    const uint32_t cyc = c.window * c.W;
     size_t off = 0;
     for (size_t d = 0; d < ctx->designs.size(); ++d) {
         Design *D = ctx->designs[d];
@@ -1072,6 +1225,8 @@ int rtlfs_create(rtlfs_ctx **out, int device) {
         CU(cudaDeviceGetAttribute(&ctx->n_sm, cudaDevAttrMultiProcessorCount, device));
         CU(cudaStreamCreateWithFlags(&ctx->s_main, cudaStreamNonBlocking));
         CU(cudaStreamCreateWithFlags(&ctx->s_heavy, cudaStreamNonBlocking));
+        for (auto &x : ctx->s_tier) CU(cudaStreamCreateWithFlags(&x, cudaStreamNonBlocking));
+        for (auto &e : ctx->ev_pk) CU(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
         // the good trace of the next window gates every fault of that window: its CTAs
         // take free SMs before pending light or heavy CTAs
         int lo_prio = 0, hi_prio = 0;
@@ -1101,6 +1256,7 @@ void rtlfs_destroy(rtlfs_ctx *ctx) {
     cudaSetDevice(ctx->device);
     if (ctx->s_main) cudaStreamSynchronize(ctx->s_main);
     if (ctx->s_heavy) cudaStreamSynchronize(ctx->s_heavy);
+    for (auto &x : ctx->s_tier) if (x) cudaStreamSynchronize(x);
     for (Design *D : ctx->designs) delete D;
     ctx->designs.clear();
     for (auto &e : ctx->ev) if (e) cudaEventDestroy(e);
@@ -1115,6 +1271,8 @@ void rtlfs_destroy(rtlfs_ctx *ctx) {
     if (ctx->s_good) { cudaStreamSynchronize(ctx->s_good); cudaStreamDestroy(ctx->s_good); }
     if (ctx->s_main) cudaStreamDestroy(ctx->s_main);
     if (ctx->s_heavy) cudaStreamDestroy(ctx->s_heavy);
+    for (auto &x : ctx->s_tier) if (x) cudaStreamDestroy(x);
+    for (auto &e : ctx->ev_pk) if (e) cudaEventDestroy(e);
     if (ctx->p_cycle) { cudaFreeHost(ctx->p_cycle); cudaFreeHost(ctx->p_port); cudaFreeHost(ctx->p_det); cudaFreeHost(ctx->p_load); }
     if (ctx->p_small) cudaFreeHost(ctx->p_small);
     if (ctx->graph_exec) cudaGraphExecDestroy(ctx->graph_exec);
@@ -1209,8 +1367,11 @@ static int run_good_only(rtlfs_ctx *ctx) {
     return RTLFS_OK;
 }
 
-int rtlfs_run(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_result *const *out,
-              uint64_t *const *out_load) {
+// One campaign. packed_ok = false: the light and heavy kernels even where the packed form could
+// run. *overflow: the packed form ran out of room for register diffs.
+static int run_campaign(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_result *const *out,
+                        uint64_t *const *out_load, bool packed_ok, bool *overflow) {
+    *overflow = false;
     if (!ctx) return RTLFS_E_ARG;
     if (ctx->designs.empty()) return fail(ctx, RTLFS_E_STATE, "no design loaded");
     if (!out) return fail(ctx, RTLFS_E_ARG, "null result array");
@@ -1223,7 +1384,7 @@ int rtlfs_run(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_result *const
     const int lblock = o.light_block > 0 ? o.light_block : 128;
     const int lcap = o.light_cap > 0 ? o.light_cap - 1 : 1;
     if (lcap > 2) return fail(ctx, RTLFS_E_ARG, "light_cap must be 0..3");
-    const int hblock = o.heavy_block > 0 ? o.heavy_block : 32;
+    int hblock = o.heavy_block > 0 ? o.heavy_block : 32;
     if (lblock < 32 || lblock > 256 || (lblock & 31)) return fail(ctx, RTLFS_E_ARG, "light_block must be a multiple of 32 in 32..256");
     if (hblock < 32 || hblock > 1024 || (hblock & 31)) return fail(ctx, RTLFS_E_ARG, "heavy_block must be a multiple of 32 in 32..1024");
     if (o.good_cluster < 0 || o.good_cluster > (int)CL_MAX || (o.good_cluster > 1 && (o.good_cluster & (o.good_cluster - 1))))
@@ -1244,7 +1405,13 @@ int rtlfs_run(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_result *const
     // uploaded from the host). HEURISTIC / MLP: computed on the device after the good
     // trace -- features, score (static cone x toggle rate, or the predictor), bucket sort
     // by descending score; the top heavy_frac of the faults start in the heavy kernel.
-    const bool dev_sched = o.scheduler != RTLFS_SCHED_PLAIN && F > 0;
+    // The packed form replaces a fault as soon as it ends, and neighbours in the fault list share
+    // the op graph's lines: it takes the list order unless the predictor's was asked for or
+    // faults start as heavy ones, and does not wait for the 256 cycles of good trace that a
+    // score needs (large design over 512 cycles: 72 against 91 ms).
+    PackPlan pk = packed_ok ? plan_pack(ctx, o.heavy_form) : PackPlan{};
+    const bool scored = o.scheduler == RTLFS_SCHED_HEURISTIC ? !pk.use || o.heavy_frac > 0.f : o.scheduler != RTLFS_SCHED_PLAIN;
+    const bool dev_sched = scored && F > 0;
     const bool use_mlp = o.scheduler == RTLFS_SCHED_MLP && ctx->has_weights;
     const float hf = dev_sched ? (o.heavy_frac >= 0.f ? std::min(o.heavy_frac, 1.f) : 0.0f) : 0.f;
     const uint32_t n_heavy = (uint32_t)(hf * F);
@@ -1257,9 +1424,44 @@ int rtlfs_run(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_result *const
         if (rc != RTLFS_OK) return rc;
     }
     if (o.heavy_form < 0 || o.heavy_form > 3) return fail(ctx, RTLFS_E_ARG, "heavy_form must be 0, 1, 2 or 3");
-    rc = ensure_heavy_scratch(ctx, hblock, o.heavy_ctas, o.heavy_form);
-    if (rc != RTLFS_OK) return rc;
     rc = prepare_good(ctx);
+    if (rc != RTLFS_OK) return rc;
+    uint32_t Tmax = 0, max_net = 0;
+    for (Design *D : ctx->designs) { Tmax = std::max(Tmax, D->T); max_net = std::max(max_net, D->n_net); }
+    // Windowed campaign: every live fault advances through the same window of cycles. The
+    // caller's windows (WU) bound the stops; the packed form runs shorter ones, also for the
+    // one-pass form, whose faults otherwise wait for the whole good trace.
+    const uint32_t WU = o.window > 0 ? (uint32_t)o.window : 0;
+    const uint32_t W = pk.use ? pack_window(WU, Tmax) : WU;
+    const uint32_t nw = W ? (Tmax + W - 1) / W : 0;
+    size_t n32 = 0, n64 = 0;   // counters of the windowed form
+    if (W && nw > 1 && !o.good_first) {
+        // SMs for the good trace of the next window while a window's faults are simulated
+        uint32_t good_ctas = ctx->gl.n_smem + ctx->gl.n_glob;
+        for (int lc = 1; lc < 5; ++lc) good_ctas += ctx->gl.n_cl[lc] << lc;
+        pk.grid = std::max(1, ctx->n_sm - (int)std::min<uint32_t>(good_ctas, (uint32_t)ctx->n_sm / 4));
+    }
+    if (pk.use) {
+        const size_t Fn = std::max<size_t>(F, 1);
+        for (auto &b : ctx->pk_items) CU(b.reserve(Fn));
+        // a tier but the last hands a fault on once, with at most its buffer's register diffs
+        // (beyond that only what a checkpoint brings: once per tier)
+        ctx->pk_prom_cap = std::min<uint64_t>((uint64_t)Fn * PACK_RPL * 41, (uint64_t)64 << 20) +
+                           (o.resume ? PACK_TIERS * ctx->ck.pool_r.size() : 0);
+        CU(ctx->pk_prom_r.reserve(ctx->pk_prom_cap));
+        CU(ctx->pk_prom_v.reserve(ctx->pk_prom_cap));
+        CU(ctx->pk_cls.reserve(Fn));
+    }
+    // behind the packed kernel the heavy kernel only takes the few faults no tier can hold
+    // for the rest of a window: cones of thousands of nodes, so 128 threads a fault unless the
+    // caller says (no-drop case of 10k nodes: 165 against 185 ms with one warp; designs whose node
+    // bitmap crowds shared memory keep the one-warp forms)
+    if (pk.use && o.heavy_block <= 0) {
+        uint32_t mnode = 0;
+        for (Design *D : ctx->designs) mnode = std::max(mnode, D->N);
+        if (mnode <= 400000) hblock = 128;
+    }
+    rc = ensure_heavy_scratch(ctx, hblock, o.heavy_ctas > 0 || !pk.use ? o.heavy_ctas : 2 * ctx->n_sm, o.heavy_form);
     if (rc != RTLFS_OK) return rc;
     uint32_t *cinit = reinterpret_cast<uint32_t *>(ctx->p_small + 10);
     cinit[0] = n_heavy; cinit[1] = 0; cinit[2] = 0; cinit[3] = 0;
@@ -1296,11 +1498,6 @@ int rtlfs_run(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_result *const
     cudaEvent_t *ev = ctx->ev;
     uint32_t launches = 0;
 
-    // Windowed campaign: every live fault advances through the same window of cycles.
-    uint32_t Tmax = 0, max_net = 0;
-    for (Design *D : ctx->designs) { Tmax = std::max(Tmax, D->T); max_net = std::max(max_net, D->n_net); }
-    const uint32_t W = o.window > 0 ? (uint32_t)o.window : 0;
-    const uint32_t nw = W ? (Tmax + W - 1) / W : 0;
     if (W) {
         const size_t Fn = std::max<size_t>(F, 1);
         uint32_t mr = 1;
@@ -1318,39 +1515,55 @@ int rtlfs_run(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_result *const
         CU(ctx->w_pool_v0.reserve(pool_cap));
         CU(ctx->w_pool_v1.reserve(pool_cap));
         ctx->w_pool_cap = pool_cap;
-        CU(ctx->w_cnt32.reserve(3 * (size_t)nw + 4));   // n_live, prom_end, n_carry | prom_total, n_light, zero
-        CU(ctx->w_cnt64.reserve(3 * (size_t)nw + 1));   // pool_top, light head, heavy head
-        while (ctx->ev_win.size() < 4 * (size_t)nw) {
+        if (pk.use)
+            for (int k = 0; k < PACK_TIERS - 2; ++k)
+                for (int b = 0; b < 2; ++b) {
+                    CU(ctx->pk_carry[k][b].reserve(Fn));
+                    CU(ctx->pk_pool_r[k][b].reserve(pool_cap));
+                    CU(ctx->pk_pool_v[k][b].reserve(pool_cap));
+                }
+        if (pk.use) {
+            CU(ctx->pk_last_r.reserve(pool_cap));
+            CU(ctx->pk_last_v.reserve(pool_cap));
+        }
+        // n_live, prom_end, n_carry | prom_total, n_light, zero | packed (pk32): prom_end from the
+        // third tier to the heavy kernel, their n_carry | items of each tier
+        n32 = (3 + 2 * (PACK_TIERS - 1)) * (size_t)nw + 4 + PACK_TIERS;
+        CU(ctx->w_cnt32.reserve(n32));
+        // pool_top, light head, heavy head | packed (pk64): pool_top and head from the third tier to
+        // the heavy kernel | promotion pool top
+        n64 = (3 + 2 * (PACK_TIERS - 1)) * (size_t)nw + 2;
+        CU(ctx->w_cnt64.reserve(n64));
+        while (ctx->ev_win.size() < 2 * WIN_TIMED * nw) {
             cudaEvent_t e;
             CU(cudaEventCreate(&e));
             ctx->ev_win.push_back(e);
         }
         uint32_t *ci = reinterpret_cast<uint32_t *>(ctx->p_small + 10);
         ci[0] = n_heavy;        // prom_total starts after the initial heavy items
-        ci[1] = F - n_heavy;    // faults in the first light window
+        ci[1] = pk.use ? F : F - n_heavy;   // faults in the first light window
         ci[2] = 0;
         ci[3] = 0;
     }
     // Checkpoint options: the campaign runs windows [w_begin, w_end).
     const bool stopping = o.stop_cycle > 0, resuming = o.resume != 0;
     if (o.stop_cycle < 0) return fail(ctx, RTLFS_E_ARG, "stop_cycle must not be negative");
-    if ((stopping || resuming) && (!W || o.use_graph))
+    if ((stopping || resuming) && (!WU || o.use_graph))
         return fail(ctx, RTLFS_E_ARG, "stop_cycle and resume need the windowed form without graph replay");
-    if (stopping && ((uint32_t)o.stop_cycle % W != 0 || (uint32_t)o.stop_cycle >= Tmax))
+    if (stopping && ((uint32_t)o.stop_cycle % WU != 0 || (uint32_t)o.stop_cycle >= Tmax))
         return fail(ctx, RTLFS_E_ARG, "stop_cycle must be a multiple of window below the longest stimulus");
     const uint32_t w_end = stopping ? (uint32_t)o.stop_cycle / W : nw;
     uint32_t w_begin = 0;
     if (resuming) {
-        int rc2 = checkpoint_matches(ctx, ctx->ck, W, nodrop, lcap);
+        int rc2 = checkpoint_matches(ctx, ctx->ck, WU, nodrop, lcap);
         if (rc2 != RTLFS_OK) return rc2;
-        w_begin = ctx->ck.window;
+        w_begin = (uint32_t)((uint64_t)ctx->ck.window * WU / W);
         if (w_begin >= w_end) return fail(ctx, RTLFS_E_ARG, "stop_cycle is not after the checkpoint");
         if (ctx->ck.pool_r.size() > ctx->w_pool_cap) return fail(ctx, RTLFS_E_ARG, "checkpoint pool exceeds capacity");
     }
     // Per-window kernel times: plain event records, or, while the campaign is captured into
     // a graph, event-record nodes of the graph itself (external records), which keep their
     // timestamps on every replay.
-    const bool timed_windows = W != 0;
     const bool good_first = W && o.good_first && !stopping && !resuming;
     auto rec_time = [&](cudaEvent_t e, cudaStream_t s) -> cudaError_t {
         return o.use_graph ? cudaEventRecordWithFlags(e, s, cudaEventRecordExternal) : cudaEventRecord(e, s);
@@ -1364,6 +1577,25 @@ int rtlfs_run(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_result *const
         f.act = ctx->d_act.p;
         f.act_stride = act_stride;
     }
+
+    // What the packed kernel's launches share.
+    const DevDesign pack_d0 = dev_view(*ctx->designs[0]);
+    auto pack_args = [&]() {
+        PackArgs pa{};
+        pa.prom_r_in = pa.prom_r = ctx->pk_prom_r.p;
+        pa.prom_v_in = pa.prom_v = ctx->pk_prom_v.p;
+        pa.prom_cap = ctx->pk_prom_cap;
+        pa.pool_cap = ctx->w_pool_cap;
+        pa.cls = ctx->pk_cls.p;
+        pa.cap_regs = (uint32_t)LIGHT_CAPS[lcap][0];
+        pa.cap_evals = (uint32_t)LIGHT_CAPS[lcap][2];
+        pa.budget_hit = ctx->d_heads.p + 3;
+        pa.fault_budget = o.fault_budget;
+        pa.counters_light = ctx->d_heads.p + 4;
+        pa.counters_heavy = ctx->d_heads.p + 6;
+        pa.err = ctx->d_err.p;
+        return pa;
+    };
 
     // Windowed stream work (good trace on s_good, light on s_main, heavy on s_heavy).
     auto enqueue_windowed = [&]() -> int {
@@ -1379,21 +1611,34 @@ int rtlfs_run(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_result *const
             CU(cudaMemsetAsync(ctx->d_cycle.p, 0xFF, (size_t)F * sizeof(int32_t), ctx->s_main));
             CU(cudaMemsetAsync(ctx->d_port.p, 0xFF, (size_t)F * sizeof(int32_t), ctx->s_main));
         }
-        CU(cudaMemsetAsync(c32, 0, (3 * (size_t)nw + 4) * sizeof(uint32_t), ctx->s_main));
-        CU(cudaMemsetAsync(c64, 0, (3 * (size_t)nw + 1) * sizeof(unsigned long long), ctx->s_main));
+        CU(cudaMemsetAsync(c32, 0, n32 * sizeof(uint32_t), ctx->s_main));
+        CU(cudaMemsetAsync(c64, 0, n64 * sizeof(unsigned long long), ctx->s_main));
         CU(cudaMemcpyAsync(prom_total, ctx->p_small + 10, 2 * sizeof(uint32_t), cudaMemcpyHostToDevice, ctx->s_main));
         CU(cudaMemsetAsync(ctx->d_err.p, 0, sizeof(uint32_t), ctx->s_main));
         if (F && !resuming) {
             CU(cudaMemsetAsync(ctx->d_load.p, 0, (size_t)F * sizeof(uint64_t), ctx->s_main));
             CU(cudaMemsetAsync(ctx->w_st_nreg.p, 0, F, ctx->s_main));
         }
+        if (pk.use && F) CU(cudaMemsetAsync(ctx->pk_cls.p, 0, F, ctx->s_main));
         if (resuming) {
             int r4 = restore_checkpoint(ctx, nw, w_begin, prom_total);
             if (r4 != RTLFS_OK) return r4;
+            if (pk.use && F) {   // the carried faults count as heavy
+                std::vector<uint8_t> cls(F, 0);
+                for (const HeavyCarry &x : ctx->ck.carry) cls[x.fault] = 1;
+                CU(cudaStreamSynchronize(ctx->s_main));
+                CU(cudaMemcpy(ctx->pk_cls.p, cls.data(), F, cudaMemcpyHostToDevice));
+            }
         }
         CU(cudaEventRecord(ctx->ev_wl, ctx->s_main));
         CU(cudaStreamWaitEvent(ctx->s_good, ctx->ev_wl, 0));
+        cudaStream_t s_hv = pk.use ? ctx->s_tier[PACK_TIERS - 3] : ctx->s_heavy;   // the heavy kernel's stream
         CU(cudaStreamWaitEvent(ctx->s_heavy, ctx->ev_wl, 0));
+        if (pk.use)
+            for (auto &x : ctx->s_tier) CU(cudaStreamWaitEvent(x, ctx->ev_wl, 0));
+        constexpr int PT = PACK_TIERS - 1;   // tiers after the first, or after the second with the heavy kernel
+        uint32_t *pk32 = c32 + 3 * (size_t)nw + 4;
+        unsigned long long *pk64 = c64 + 3 * (size_t)nw + 1;
         const uint32_t lblocks = (uint32_t)std::max<int64_t>(1, std::min<int64_t>(((int64_t)F + lblock - 1) / lblock,
                                                                                   (int64_t)lgrid_cap));
         // The scheduler of the first window reads the toggle rates of the first TOGGLE_CYCLES
@@ -1461,13 +1706,73 @@ int rtlfs_run(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_result *const
             wl.budget_hit = ctx->d_heads.p + 3;
             wl.fault_budget = o.fault_budget;
             wl.counters = ctx->d_heads.p + 4;
-            if (timed_windows) CU(rec_time(ctx->ev_win[0 * nw + w], ctx->s_main));
-            if (F) { CU(launch_light_window(ctx->d_designs.p, f, wl, lcap, lblock, (int)lblocks, ctx->s_main)); ++launches; }
-            if (timed_windows) CU(rec_time(ctx->ev_win[1 * nw + w], ctx->s_main));
-            CU(cudaMemcpyAsync(c32 + nw + w, prom_total, sizeof(uint32_t), cudaMemcpyDeviceToDevice, ctx->s_main));
-            CU(cudaEventRecord(ctx->ev_wl, ctx->s_main));
+            if (!pk.use) CU(rec_time(ctx->ev_win[0 * nw + w], ctx->s_main));
+            if (pk.use) {
+                // first tier on s_main, second on s_heavy, the others on s_tier (the heavy kernel
+                // behind the last): each takes what the tier before handed on in this window
+                PackArgs pa = pack_args();
+                pa.t0 = t0; pa.t1 = t1;
+                pa.prom_total = prom_total;
+                pa.prom_top = pk64 + 2 * PT * nw;
+                const int in = w & 1 ? 0 : 1, out = w & 1;   // window parity of the ping-pong buffers
+                for (int tier = 0; tier < PACK_TIERS && F; ++tier) {
+                    PackArgs p = pa;
+                    p.tier_evals = pk.evals[tier];
+                    p.items_out = ctx->pk_items[tier].p;
+                    p.n_items_out = pk32 + 2 * PT * nw + tier;
+                    if (tier == PACK_TIERS - 1) {   // emptied every window: its faults come back
+                        p.n_items_out = pk32 + (PT - 1) * nw + w;
+                        p.prom_r = ctx->pk_last_r.p; p.prom_v = ctx->pk_last_v.p;
+                        p.prom_top = pk64 + (PT - 1) * nw + w;
+                        p.prom_cap = ctx->w_pool_cap;
+                    }
+                    cudaStream_t st = tier == 0 ? ctx->s_main : tier == 1 ? ctx->s_heavy : ctx->s_tier[tier - 2];
+                    if (tier == 0) {
+                        p.live_in = w == 0 ? ctx->d_order.p : wl.live_in;
+                        p.n_live_in = wl.n_live_in; p.reverse = wl.reverse;
+                        p.fresh = w == 0; p.n_heavy = n_heavy;
+                        p.head = wl.head;
+                        p.live_out = wl.live_out; p.n_live_out = wl.n_live_out;
+                        p.st_nreg = wl.st_nreg; p.st_r = wl.st_r; p.st_v = wl.st_v;
+                    } else {
+                        const int k = tier - 2;   // buffers of the third tier on
+                        HeavyCarry *car[2] = {tier == 1 ? ctx->w_carry0.p : ctx->pk_carry[k][0].p, tier == 1 ? ctx->w_carry1.p : ctx->pk_carry[k][1].p};
+                        uint32_t *pr[2] = {tier == 1 ? ctx->w_pool_r0.p : ctx->pk_pool_r[k][0].p, tier == 1 ? ctx->w_pool_r1.p : ctx->pk_pool_r[k][1].p};
+                        uint64_t *pv[2] = {tier == 1 ? ctx->w_pool_v0.p : ctx->pk_pool_v[k][0].p, tier == 1 ? ctx->w_pool_v1.p : ctx->pk_pool_v[k][1].p};
+                        uint32_t *ncar = tier == 1 ? c32 + 2 * nw : pk32 + (PT + k) * nw;
+                        uint32_t *end = tier == 1 ? c32 + nw : pk32 + k * nw;
+                        p.carry_in = car[in]; p.pool_r_in = pr[in]; p.pool_v_in = pv[in];
+                        p.carry_out = car[out]; p.pool_r = pr[out]; p.pool_v = pv[out];
+                        p.n_carry_in = w == 0 ? zero : ncar + (w - 1);
+                        p.n_carry_out = ncar + w;
+                        p.pool_top = (tier == 1 ? c64 : pk64 + k * nw) + w;
+                        p.head = (tier == 1 ? c64 + 2 * nw : pk64 + (PT + k) * nw) + w;
+                        p.items = ctx->pk_items[tier - 1].p;
+                        p.item_begin = w == 0 ? zero : end + (w - 1);
+                        p.item_end = end + w;
+                        CU(cudaStreamWaitEvent(st, ctx->ev_pk[tier - 1], 0));
+                    }
+                    CU(rec_time(ctx->ev_win[2 * tier * (size_t)nw + w], st));
+                    CU(launch_pack(tier, pk.multi, ctx->d_designs.p, pack_d0, f, p, pk.warps[tier], pk.grid, st));
+                    ++launches;
+                    CU(rec_time(ctx->ev_win[(2 * tier + 1) * (size_t)nw + w], st));
+                    if (tier + 1 < PACK_TIERS)
+                        CU(cudaMemcpyAsync((tier == 0 ? c32 + nw : pk32 + (tier - 1) * nw) + w, p.n_items_out, sizeof(uint32_t),
+                                           cudaMemcpyDeviceToDevice, st));
+                    CU(cudaEventRecord(ctx->ev_pk[tier], st));
+                }
+            } else if (F) {
+                CU(launch_light_window(ctx->d_designs.p, f, wl, lcap, lblock, (int)lblocks, ctx->s_main));
+                ++launches;
+            }
+            if (!pk.use) {
+                CU(rec_time(ctx->ev_win[1 * nw + w], ctx->s_main));
+                CU(cudaMemcpyAsync(c32 + nw + w, prom_total, sizeof(uint32_t), cudaMemcpyDeviceToDevice, ctx->s_main));
+                CU(cudaEventRecord(ctx->ev_wl, ctx->s_main));
+                CU(cudaStreamWaitEvent(ctx->s_heavy, ctx->ev_wl, 0));
+            }
             // heavy kernel of the window: carried heavy faults plus this window's promotions
-            CU(cudaStreamWaitEvent(ctx->s_heavy, ctx->ev_wl, 0));
+            // (packed: the faults the packed warps gave up, from the start of the window)
             WinHeavy wh{};
             wh.carry_in = (w & 1) ? ctx->w_carry0.p : ctx->w_carry1.p;
             wh.n_carry_in = w == 0 ? zero : c32 + 2 * nw + (w - 1);
@@ -1489,16 +1794,36 @@ int rtlfs_run(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_result *const
             wh.fault_budget = o.fault_budget;
             wh.counters = ctx->d_heads.p + 6;
             wh.err = ctx->d_err.p;
-            if (timed_windows) CU(rec_time(ctx->ev_win[2 * nw + w], ctx->s_heavy));
-            CU(launch_heavy_window(ctx->d_designs.p, f, wh, hs, hblock, hgrid, ctx->s_heavy));
+            if (pk.use) {   // the faults the last tier handed on, to the end of the window only:
+                const int out = w & 1, k = PT - 1;   // its survivors go back to the last tier's list
+                wh.carry_out = ctx->pk_carry[k - 1][out].p;
+                wh.pool_r_out = ctx->pk_pool_r[k - 1][out].p; wh.pool_v_out = ctx->pk_pool_v[k - 1][out].p;
+                wh.n_carry_in = zero;
+                wh.n_carry_out = pk32 + (PT + k - 1) * nw + w;
+                wh.pool_top_out = pk64 + (k - 1) * nw + w;
+                wh.pitems = ctx->pk_items[PACK_TIERS - 1].p;
+                wh.prom_r = ctx->pk_last_r.p; wh.prom_v = ctx->pk_last_v.p;
+                wh.prom_begin = zero;
+                wh.prom_end = pk32 + k * nw + w;
+                wh.head = pk64 + (PT + k) * nw + w;
+            }
+            const size_t tk = pk.use ? PACK_TIERS : 1;   // its timed slot
+            CU(rec_time(ctx->ev_win[2 * tk * nw + w], s_hv));
+            CU(launch_heavy_window(ctx->d_designs.p, f, wh, hs, hblock, hgrid, s_hv));
             ++launches;
-            if (timed_windows) CU(rec_time(ctx->ev_win[3 * nw + w], ctx->s_heavy));
+            CU(rec_time(ctx->ev_win[(2 * tk + 1) * nw + w], s_hv));
         }
         CU(cudaEventRecord(ev[2], ctx->s_main));
         if (o.use_graph) CU(rec_time(ctx->ev_gend, ctx->s_good));
         CU(cudaEventRecord(ev[3], ctx->s_good));
         CU(cudaStreamWaitEvent(ctx->s_main, ev[3], 0));
-        CU(cudaEventRecord(ev[4], ctx->s_heavy));
+        if (pk.use) {
+            for (int tier = 1; tier + 1 < PACK_TIERS; ++tier) {
+                CU(cudaEventRecord(ctx->ev_pk[tier], tier == 1 ? ctx->s_heavy : ctx->s_tier[tier - 2]));
+                CU(cudaStreamWaitEvent(ctx->s_main, ctx->ev_pk[tier], 0));
+            }
+        }
+        CU(cudaEventRecord(ev[4], s_hv));
         CU(cudaStreamWaitEvent(ctx->s_main, ev[4], 0));
         if (F) {
             CU(cudaMemcpyAsync(ctx->p_cycle, ctx->d_cycle.p, (size_t)F * 4, cudaMemcpyDeviceToHost, ctx->s_main));
@@ -1574,7 +1899,8 @@ int rtlfs_run(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_result *const
         std::vector<uint64_t> key = {F, n_heavy, ql.n_light, (uint64_t)lcap, (uint64_t)lblock,
                                      (uint64_t)lgrid, (uint64_t)hblock, (uint64_t)hgrid,
                                      (uint64_t)dev_sched, (uint64_t)use_mlp, o.fault_budget, W,
-                                     (uint64_t)nodrop, (uint64_t)good_first, (uint64_t)o.order_classes};
+                                     (uint64_t)nodrop, (uint64_t)good_first, (uint64_t)o.order_classes,
+                                     (uint64_t)pk.use, (uint64_t)pk.grid};
         const void *ptrs[] = {ctx->d_designs.p, ctx->d_list_smem.p, ctx->d_list_glob.p, ctx->d_order.p, ctx->d_err.p, ctx->h_gbm.p,
                               ctx->d_init_items.p, ctx->d_prom_items.p, ctx->d_heads.p, ctx->d_counters.p,
                               ctx->d_load.p, ctx->d_cycle.p, ctx->d_port.p, ctx->d_det.p, ctx->d_site.p,
@@ -1585,8 +1911,12 @@ int rtlfs_run(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_result *const
                               ctx->w_st_v.p, ctx->w_live0.p, ctx->w_live1.p, ctx->w_cnt32.p, ctx->w_cnt64.p,
                               ctx->w_carry0.p, ctx->w_carry1.p, ctx->w_pool_r0.p, ctx->w_pool_r1.p,
                               ctx->d_fport.p, ctx->d_ft0.p, ctx->d_mism.p,
-                              ctx->w_pool_v0.p, ctx->w_pool_v1.p, ctx->d_act.p};
+                              ctx->w_pool_v0.p, ctx->w_pool_v1.p, ctx->d_act.p, ctx->pk_prom_r.p, ctx->pk_prom_v.p, ctx->pk_cls.p,
+                              ctx->pk_items[0].p, ctx->pk_items[1].p, ctx->pk_items[2].p, ctx->pk_items[3].p, ctx->pk_last_r.p, ctx->pk_last_v.p};
         for (const void *q : ptrs) key.push_back((uint64_t)(uintptr_t)q);
+        for (int k = 0; k < 2 * (PACK_TIERS - 2); ++k)
+            key.insert(key.end(), {(uint64_t)(uintptr_t)ctx->pk_carry[k >> 1][k & 1].p, (uint64_t)(uintptr_t)ctx->pk_pool_r[k >> 1][k & 1].p,
+                                   (uint64_t)(uintptr_t)ctx->pk_pool_v[k >> 1][k & 1].p});
         const GoodLaunch &g = ctx->gl;
         key.insert(key.end(), {g.n_smem, g.n_glob, g.max_net_s, g.max_reg_s, g.max_ch_s, g.max_ch_g,
                                ctx->hs_net, ctx->hs_reg, ctx->hs_node, ctx->hs_lv, (uint64_t)ctx->heavy_exact, (uint64_t)ctx->heavy_gbm,
@@ -1623,6 +1953,7 @@ int rtlfs_run(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_result *const
     CU(cudaStreamSynchronize(ctx->s_main));
     {
         const uint32_t kerr = *reinterpret_cast<const uint32_t *>(ctx->p_small + 12);
+        *overflow = pk.use && (kerr & 2u);
         if (kerr & 2u)
             return fail(ctx, RTLFS_E_NOMEM, "heavy register-diff pool overflowed; run with window = 0");
         if (kerr & 1u)
@@ -1636,7 +1967,7 @@ int rtlfs_run(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_result *const
     ctx->mism_valid = nodrop && !stopping;
     std::vector<uint8_t> pending;
     if (stopping) {
-        rc = take_checkpoint(ctx, nw, w_end, W, nodrop, lcap, &pending);
+        rc = take_checkpoint(ctx, nw, w_end, W, WU, nodrop, lcap, pk.use, &pending);
         if (rc != RTLFS_OK) return rc;
     } else {
         ctx->ck.valid = false;   // the campaign ran to its end
@@ -1645,14 +1976,17 @@ int rtlfs_run(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_result *const
     // Scatter results and counters.
     rtlfs_stats &st = ctx->stats;
     st = rtlfs_stats{};
+    auto window_times = [&]() {   // first tier or light kernel; the others
+        for (uint32_t w = w_begin; w < w_end; ++w)
+            for (size_t k = 0; k < (pk.use ? WIN_TIMED : 2); ++k)
+                if (F || !pk.use || k == PACK_TIERS)
+                    (k == 0 ? st.light_ms : st.heavy_ms) += ev_ms(ctx->ev_win[2 * k * nw + w], ctx->ev_win[(2 * k + 1) * nw + w]);
+    };
     if (o.use_graph && W) {   // whole campaign, good-trace stream and each window kernel
         st.total_ms = ev_ms(ctx->ev_graph[0], ctx->ev_graph[1]);
         st.good_ms = ev_ms(ctx->ev_graph[0], ctx->ev_gend);
         st.prep_ms = std::chrono::duration<double, std::milli>(t_host1 - t_host0).count();
-        for (uint32_t w = w_begin; w < w_end; ++w) {
-            st.light_ms += ev_ms(ctx->ev_win[w], ctx->ev_win[nw + w]);
-            st.heavy_ms += ev_ms(ctx->ev_win[2 * nw + w], ctx->ev_win[3 * nw + w]);
-        }
+        window_times();
     } else if (o.use_graph) {   // whole campaign only; per-phase times are not available
         st.total_ms = ev_ms(ctx->ev_graph[0], ctx->ev_graph[1]);
         st.prep_ms = std::chrono::duration<double, std::milli>(t_host1 - t_host0).count();
@@ -1660,10 +1994,7 @@ int rtlfs_run(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_result *const
         st.total_ms = ev_ms(ev[0], ev[5]);
         st.good_ms = ev_ms(ev[0], ev[3]);
         st.prep_ms = std::chrono::duration<double, std::milli>(t_host1 - t_host0).count();
-        for (uint32_t w = w_begin; w < w_end; ++w) {
-            st.light_ms += ev_ms(ctx->ev_win[w], ctx->ev_win[nw + w]);
-            st.heavy_ms += ev_ms(ctx->ev_win[2 * nw + w], ctx->ev_win[3 * nw + w]);
-        }
+        window_times();
         st.faulty_ms = ev_ms(ev[1], ev[4]);
     } else {
         st.total_ms = ev_ms(ev[0], ev[5]);
@@ -1680,7 +2011,7 @@ int rtlfs_run(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_result *const
         st.promoted = cnts[0] - st.heavy_initial;
     }
     st.n_launches = launches;
-    st.heavy_form = ctx->heavy_gbm ? 3u : ctx->heavy_exact ? 1u : 2u;
+    st.heavy_form = pk.use ? 4u : ctx->heavy_gbm ? 3u : ctx->heavy_exact ? 1u : 2u;
     st.light_evals = heads[4];
     st.light_fault_cycles = heads[5];
     st.heavy_evals = heads[6];
@@ -1709,6 +2040,13 @@ int rtlfs_run(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_result *const
     if (heads[3]) return fail(ctx, RTLFS_E_TIMEOUT, "%llu faults ran out of their work budget", heads[3]);
     ctx->err.clear();
     return RTLFS_OK;
+}
+
+int rtlfs_run(rtlfs_ctx *ctx, const rtlfs_run_opts *opts, rtlfs_result *const *out, uint64_t *const *out_load) {
+    bool overflow = false;
+    const int rc = run_campaign(ctx, opts, out, out_load, true, &overflow);
+    // more register diffs than the packed form's pools hold: the light and heavy kernels
+    return overflow ? run_campaign(ctx, opts, out, out_load, false, &overflow) : rc;
 }
 
 int rtlfs_run_plain(rtlfs_ctx *ctx, rtlfs_result *const *out) {

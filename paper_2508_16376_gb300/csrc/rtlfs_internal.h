@@ -49,6 +49,13 @@ struct DevDesign {
     const uint32_t *fo_off;     // [n_net + 1] fan-out CSR: consumer node indices
     const uint32_t *fo_idx;     // [n_fo]
     const uint16_t *fo_lvl;     // [n_fo] level of each consumer
+    // Packed kernel. An edge: consumer net | operands it feeds << 27 (bit 0, 1: value slots 0, 1;
+    // bit 2: MUX2 select); value slots: operands a and b, or b and c of a MUX2.
+    const uint32_t *fo_edge;    // [n_fo] edges in fo_idx order
+    const uint4    *rec;        // [n_net][8] {nets of value slot 0, slot 1, select, meta (CONST: as desc)
+                                // | the slots the op reads << 4 | PM_*}, netinfo (z: the dreg_rec itself
+                                // when it is the only one), the first eight edges (2 x uint4), their
+                                // levels << 4 (8 x u16), unused: one 128-byte line per net
     const uint32_t *dreg_off;   // [n_net + 1] registers latching each net
     const uint32_t *dreg_idx;   // [n_dreg]
     const uint32_t *dreg_rec;   // [n_dreg] register index | register width << 25
@@ -68,6 +75,10 @@ struct DevDesign {
     const uint4    *cl_reg;     // {register, D location, width, D net} by home CTA
     const uint32_t *cl_reg_off; // [C + 1] registers of each CTA (a contiguous index range)
 };
+
+// Evaluation masks of a packed record's meta (pack_eval).
+constexpr uint32_t PM_LEFT = 1u << 24, PM_SUM = 1u << 25, PM_CMP = 1u << 26;
+constexpr uint32_t PM_A = 1u << 28, PM_B = 1u << 29, PM_C = 1u << 30, PM_D = 1u << 31;
 
 // A net's location for the cluster good trace, 32 bits: the word in the holding CTA's
 // value area (node values [0, own), register banks [own, own + 2 rown), inputs after
@@ -118,6 +129,12 @@ struct HeavyItem {
     uint32_t nreg;
     uint32_t reg_r[LIGHT_KR];
     uint64_t reg_v[LIGHT_KR];
+};
+
+// A fault handed on by the packed kernel: resume at cycle t with `nreg` register diffs at
+// off in the promotion pool.
+struct PackItem {
+    uint32_t fault, t, nreg, off;
 };
 
 struct Queues {
@@ -207,6 +224,9 @@ struct WinHeavy {
     unsigned long long *pool_top_out;
     uint64_t pool_cap;
     const HeavyItem *prom;        // this window's promotions: prom[*prom_begin .. *prom_end)
+    const PackItem *pitems;       // not null: they are these, with their pool
+    const uint32_t *prom_r;
+    const uint64_t *prom_v;
     const uint32_t *prom_begin;
     const uint32_t *prom_end;
     unsigned long long *head;
@@ -216,6 +236,63 @@ struct WinHeavy {
     unsigned long long *counters;
     uint32_t *err;                // bit 1: pool overflow
 };
+
+// ---- packed kernel (rtlfs_pack.cu): several faults per warp, one level of each per round ----
+constexpr int PACK_TIERS = 4;            // one, several and 32 lanes per fault, and a CTA
+constexpr int PACK_RPL = 4;              // register diffs per lane
+constexpr int PACK_MAX_WARPS = 16;       // warps per CTA the register allocation allows
+constexpr uint32_t PACK_NETS = 1u << 27;
+constexpr uint32_t PACK_LEVELS = 4095;   // levels a 16-bit tag can name beside a place below 16
+
+struct PackArgs {
+    // queue: carried faults (back to front), then the live list (first tier) or the faults
+    // promoted in this window (items [*item_begin, *item_end))
+    const HeavyCarry *carry_in;
+    const uint32_t *n_carry_in;   // null: none
+    const uint32_t *pool_r_in;
+    const uint64_t *pool_v_in;
+    const uint32_t *live_in;      // null: items
+    const uint32_t *n_live_in;    // null: n_live of them
+    uint32_t n_live, reverse;     // reverse: take live_in back to front
+    uint32_t fresh, n_heavy;      // fresh: no state yet, and the first n_heavy count as heavy
+    const PackItem *items;
+    const uint32_t *item_begin, *item_end;   // item_begin null: 0
+    const uint32_t *prom_r_in;
+    const uint64_t *prom_v_in;
+    unsigned long long *head;
+    uint32_t t0, t1;              // cycles [t0, min(t1, T)) (items: from their own cycle)
+    // survivors at t1: the first tier's with their register diffs in st_*, else in the pool
+    uint32_t *live_out, *n_live_out;
+    uint8_t *st_nreg;             // [F]
+    uint32_t *st_r;               // [LIGHT_KR][F]
+    uint64_t *st_v;               // [LIGHT_KR][F]
+    HeavyCarry *carry_out;
+    uint32_t *n_carry_out;
+    uint32_t *pool_r;
+    uint64_t *pool_v;
+    unsigned long long *pool_top;
+    uint64_t pool_cap;
+    // faults handed to the next tier
+    PackItem *items_out;
+    uint32_t *n_items_out;
+    uint32_t *prom_r;
+    uint64_t *prom_v;
+    unsigned long long *prom_top;
+    uint64_t prom_cap;
+    uint8_t *cls;                 // [F] 1: the fault counts as heavy
+    uint32_t tier_evals;          // a fault with more evaluations in a cycle goes to the next tier
+    uint32_t cap_regs, cap_evals; // a light fault beyond these in a cycle counts as heavy
+    uint32_t *prom_total;         // light faults that became heavy
+    unsigned long long *budget_hit;
+    uint64_t fault_budget;
+    unsigned long long *counters_light, *counters_heavy;   // [0] evaluations, [1] fault-cycles
+    uint32_t *err;                // bit 1: pool overflow
+};
+
+size_t pack_smem_bytes(int tier, int warps);
+// d0: the design when there is only one (multi = false).
+cudaError_t launch_pack(int tier, bool multi, const DevDesign *d_designs, const DevDesign &d0, DevFaults f,
+                        const PackArgs &q, int warps, int grid, cudaStream_t stream);
 
 // Launchers (rtlfs_kernels.cu). All enqueue on `stream` and return the launch status.
 size_t good_smem_bytes(bool use_smem, uint32_t max_net, uint32_t max_reg, uint32_t max_chunks, bool staged);

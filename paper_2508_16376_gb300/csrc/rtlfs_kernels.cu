@@ -16,70 +16,13 @@
 // fault, evaluating each topological level of the cone in parallel (the few high-load
 // tasks split along their bad gates, Sec. IV-C-2). The register latch is folded into
 // the cycle loop of each fault (no separate synchronization phase, Sec. IV-D).
+#include "rtlfs_device.h"
 #include "rtlfs_internal.h"
 
 #include <climits>
 #include <cstdio>
 
 namespace rtlfs {
-
-__device__ __forceinline__ uint64_t wmask(uint32_t w) {
-    return w >= 64 ? ~0ull : ((1ull << w) - 1ull);
-}
-
-__device__ __forceinline__ int n_operands(uint32_t op) {
-    return op == OP_CONST ? 0
-         : (op == OP_NOT || op == OP_SHL || op == OP_SHR || op == OP_SLICE) ? 1
-         : op == OP_MUX2 ? 3 : 2;
-}
-
-// One word-level op on zero-extended operands, masked to the node width.
-__device__ __forceinline__ uint64_t eval_op(uint4 d, uint64_t a, uint64_t b, uint64_t c) {
-    const uint32_t m = d.w, k = meta_k(m);
-    uint64_t r;
-    switch (meta_op(m)) {
-    case OP_AND:    r = a & b; break;
-    case OP_OR:     r = a | b; break;
-    case OP_XOR:    r = a ^ b; break;
-    case OP_NOT:    r = ~a; break;
-    case OP_ADD:    r = a + b; break;
-    case OP_SUB:    r = a - b; break;
-    case OP_MUX2:   r = a ? b : c; break;
-    case OP_EQ:     r = (a == b) ? 1ull : 0ull; break;
-    case OP_LT:     r = (a < b) ? 1ull : 0ull; break;
-    case OP_SHL:    r = k >= 64 ? 0ull : (a << k); break;
-    case OP_SHR:
-    case OP_SLICE:  r = k >= 64 ? 0ull : (a >> k); break;
-    case OP_CONCAT: r = (k >= 64 ? 0ull : (a << k)) | b; break;
-    default:        r = ((uint64_t)d.y << 32) | d.x; break;   // CONST
-    }
-    return r & wmask(meta_w(m));
-}
-
-// The fault function at a fault's site (Sec. IV-A: applied wherever the site's value is
-// produced; a virtual function in the paper, a switch on the kind here): stuck-at 0 or 1
-// forces the bit in every cycle; a transient flip (an SEU on a register, an SET on an
-// input or node net) inverts it during cycle t0 only. A port fault (port != NO_PORT) acts
-// on what one output port observes of the site net and on nothing else.
-struct FaultSite {
-    uint32_t site, port, kind, t0;
-    uint64_t bm;   // one-hot mask of the faulted bit
-    __device__ __forceinline__ uint64_t apply(uint64_t v, uint32_t t) const {
-        return kind == FK_SA0 ? (v & ~bm) : kind == FK_SA1 ? (v | bm) : (t == t0 ? v ^ bm : v);
-    }
-    // whether the fault function changes anything in cycle t (a stuck-at fault: always)
-    __device__ __forceinline__ bool acts(uint32_t t) const { return kind != FK_FLIP || t == t0; }
-};
-
-__device__ __forceinline__ FaultSite load_fault(const DevFaults &f, uint32_t fid) {
-    FaultSite s;
-    s.site = f.site[fid];
-    s.kind = f.val[fid];
-    s.bm = 1ull << f.bit[fid];
-    s.port = f.port ? f.port[fid] : NO_PORT;
-    s.t0 = f.t0 ? f.t0[fid] : 0u;
-    return s;
-}
 
 // ===================================================================================
 // Good-machine trace. One CTA per design walks the cycles; inside a cycle the nodes of
@@ -546,19 +489,6 @@ __global__ void activation_kernel(const DevDesign *__restrict__ designs, DevFaul
     }
 }
 
-// First cycle in [t, tend) where the fault is active by itself, or tend.
-__device__ __forceinline__ uint32_t next_active(const uint64_t *__restrict__ fact, uint32_t t, uint32_t tend) {
-    while (t < tend) {
-        const uint64_t w = __ldg(fact + (t >> 6)) >> (t & 63u);
-        if (w) {
-            const uint32_t a = t + (uint32_t)(__ffsll((long long)w) - 1);
-            return a < tend ? a : tend;
-        }
-        t = (t | 63u) + 1;
-    }
-    return tend;
-}
-
 // ===================================================================================
 // Heavy kernel: one CTA per fault (by default a single warp). Shared memory holds a bitmap
 // over the nodes (dirty: some operand differs), the number of dirty nodes per level (so an
@@ -658,19 +588,6 @@ __device__ __forceinline__ void heavy_zero(const HeavySmem &m, const HeavyScratc
     }
     for (uint32_t i = tid; i < m.nlw; i += B) m.lvm[i] = 0;
     if (tid == 0) { V.nfr = 0; V.nl = 0; V.load = 0; }
-}
-
-// Loads issued where they stand: volatile, so the compiler does not sink them into the
-// branch that consumes them and they travel together with the operand loads.
-__device__ __forceinline__ uint32_t ld_early_u32(const uint32_t *p) {
-    uint32_t v;
-    asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(v) : "l"(p));
-    return v;
-}
-__device__ __forceinline__ uint32_t ld_early_u16(const uint16_t *p) {
-    unsigned short v;
-    asm volatile("ld.global.nc.u16 %0, [%1];" : "=h"(v) : "l"(p));
-    return v;
 }
 
 // Outcome of one heavy fault's run.
@@ -1413,15 +1330,18 @@ heavy_window_kernel(const DevDesign *__restrict__ designs, DevFaults f, WinHeavy
         const bool carried = idx < n_carry;
         // carried faults back to front: the slowest of the last window first
         const HeavyCarry cin = carried ? q.carry_in[n_carry - 1 - (uint32_t)idx] : HeavyCarry{0, 0, 0};
-        const HeavyItem &it = q.prom[pb + (carried ? 0 : idx - n_carry)];
-        const uint32_t fid = carried ? cin.fault : it.fault;
+        const uint32_t at = pb + (carried ? 0 : (uint32_t)(idx - n_carry));
+        const HeavyItem &it = q.prom[at];
+        const PackItem pi = carried ? PackItem{cin.fault, q.t0, cin.nreg, 0u}
+                          : q.pitems ? q.pitems[at] : PackItem{it.fault, it.t, it.nreg, 0u};
+        const uint32_t fid = pi.fault;
         const DevDesign &D = designs[f.design[fid]];
         const uint32_t tend = min(q.t1, D.T);   // this window ends at tend
-        const uint32_t t_start = carried ? q.t0 : it.t;
-        const uint32_t nreg0 = carried ? cin.nreg : it.nreg;
+        const uint32_t t_start = pi.t;
+        const uint32_t nreg0 = pi.nreg;
         for (uint32_t k = tid; k < nreg0; k += B) {
-            regR[k] = carried ? q.pool_r_in[cin.off + k] : it.reg_r[k];
-            regV[k] = carried ? q.pool_v_in[cin.off + k] : it.reg_v[k];
+            regR[k] = carried ? q.pool_r_in[cin.off + k] : q.pitems ? q.prom_r[pi.off + k] : it.reg_r[k];
+            regV[k] = carried ? q.pool_v_in[cin.off + k] : q.pitems ? q.prom_v[pi.off + k] : it.reg_v[k];
         }
         if (tid == 0) V.load = 0;
         hsync<WARP>();
