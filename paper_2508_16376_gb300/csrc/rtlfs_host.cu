@@ -72,6 +72,10 @@ struct Design {
     DBuf<float> d_net_static;
     DBuf<uint4> d_desc, d_netinfo, d_rec;
     DBuf<uint2> d_chunks;
+    std::vector<uint4> gdesc, gconst;   // good trace in shared memory (DevDesign)
+    DBuf<uint4> d_gdesc, d_gconst;
+    std::vector<uint32_t> gfirst;
+    DBuf<uint32_t> d_gfirst;
     DBuf<uint32_t> d_lvl_start, d_fo_off, d_fo_idx, d_fo_edge, d_dreg_off, d_dreg_idx, d_dreg_rec, d_reg_d,
         d_outport, d_out_net;
     DBuf<uint16_t> d_node_level, d_fo_lvl;
@@ -89,11 +93,11 @@ struct Design {
     bool trace_valid = false;
     // cluster good-trace plans, indexed by log2 of the cluster size (built on first use)
     struct ClusterPlan {
-        uint32_t own = 0, rown = 0, max_ch = 0;
+        uint32_t own = 0, rown = 0, steps = 0, width = 0, latch_sync = 0;
         size_t smem = 0;
         int usable = -1;   // clusters of this size can be resident (-1: not asked yet)
-        DBuf<uint4> d_desc, d_chunk, d_reg;
-        DBuf<uint32_t> d_ch_off, d_reg_off;
+        DBuf<uint4> d_desc, d_reg, d_const;
+        DBuf<uint32_t> d_reg_off, d_const_off;
     };
     std::unique_ptr<ClusterPlan> plan[5];
 };
@@ -103,6 +107,7 @@ struct Design {
 struct GoodLaunch {
     uint32_t n_smem = 0, n_glob = 0, max_net_s = 0, max_reg_s = 0, max_ch_s = 0, max_ch_g = 0;
     uint32_t n_cl[5] = {};        // designs on each cluster list (index log2 of the cluster size)
+    uint32_t thr_cl[5] = {};      // threads per CTA of each cluster launch
     size_t smem_cl[5] = {};       // shared memory per CTA of each cluster launch
 };
 
@@ -237,6 +242,35 @@ inline int n_ops(uint32_t op) {
     return op == OP_CONST ? 0
          : (op == OP_NOT || op == OP_SHL || op == OP_SHR || op == OP_SLICE) ? 1
          : op == OP_MUX2 ? 3 : 2;
+}
+
+// A node of the good trace: {nets of value slots 0 and 1, select net, GM_*}; slots that the op does
+// not read, and both of a constant, are the node's own net `self`.
+inline uint4 good_slots(uint4 d, uint32_t self) {
+    const uint32_t op = meta_op(d.w);
+    const int no = n_ops(op);
+    uint4 g = make_uint4(no >= 1 ? d.x : self, no >= 2 ? d.y : self, self, GM_VALID | (64u - meta_w(d.w)) << 8);
+    switch (op) {
+    case OP_AND: g.w |= GM_A; break;
+    case OP_OR: case OP_CONST: g.w |= GM_A | GM_B | GM_C; break;
+    case OP_XOR: g.w |= GM_B | GM_C; break;
+    case OP_NOT: g.w |= GM_B | GM_D; break;
+    case OP_ADD: g.w |= GM_SUM; break;
+    case OP_SUB: g.w |= GM_SUM | GM_NEG; break;
+    case OP_MUX2: g = make_uint4(d.y, d.z, d.x, g.w | GM_C | GM_MUX); break;
+    case OP_EQ: g.w |= GM_CMP | GM_EQ | GM_NEG; break;
+    case OP_LT: g.w |= GM_CMP | GM_NEG; break;
+    case OP_SHL: g.w |= GM_B | GM_LEFT | meta_k(d.w); break;
+    case OP_CONCAT: g.w |= GM_B | GM_C | GM_LEFT | meta_k(d.w); break;
+    default: g.w |= GM_B | meta_k(d.w); break;   // SHR, SLICE
+    }
+    return g;
+}
+
+// Value of a CONST node, {low, high word}, masked to its width.
+inline uint2 const_value(uint4 d) {
+    const uint64_t v = ((uint64_t)d.y << 32 | d.x) & (~0ull >> (64u - meta_w(d.w)));
+    return make_uint2((uint32_t)v, (uint32_t)(v >> 32));
 }
 
 inline uint64_t host_mask(uint32_t w) { return w >= 64 ? ~0ull : ((1ull << w) - 1ull); }
@@ -472,6 +506,41 @@ int build_design(rtlfs_ctx *ctx, Design &D, const rtlfs_node *nodes, uint32_t N,
             D.chunks.push_back(make_uint2(lo, hi | (hi == D.lvl_start[l + 1] ? 0x80000000u : 0u)));
         }
     }
+    // Records of the good trace in shared memory (net ids of 16 bits hold every design that fits
+    // there): a level's nodes in groups of 32, dealt to the warps in turn.
+    D.gdesc.clear();
+    D.gconst.clear();
+    D.gfirst.assign(GOOD_BLOCK / 32 + 1, 0);
+    if (n_net <= 0xFFFFu) {
+        constexpr uint32_t NW = GOOD_BLOCK / 32;
+        std::vector<std::vector<uint4>> gw(NW);
+        std::vector<uint32_t> ended(NW, 0);   // level ends that the warp's groups have counted
+        auto catch_up = [&](uint32_t k, uint32_t level) {   // the ends before `level`, on the last group
+            if (gw[k].empty() && level) gw[k].assign(32, make_uint4(0, 0, 0, 0));
+            for (size_t i = gw[k].size() - std::min<size_t>(32, gw[k].size()); i < gw[k].size(); ++i) gw[k][i].w += level - ended[k];
+            ended[k] = level;
+        };
+        uint32_t next = 0;
+        for (uint32_t l = 0; l < NL; ++l) {
+            for (uint32_t lo = D.lvl_start[l]; lo < D.lvl_start[l + 1]; lo += 32) {
+                const uint32_t k = next++ % NW;
+                catch_up(k, l);
+                for (uint32_t n = lo; n < lo + 32; ++n) {
+                    if (n >= D.lvl_start[l + 1]) { gw[k].push_back(make_uint4(0, 0, 0, 0)); continue; }
+                    const uint4 g = good_slots(D.desc[n], IR + n);
+                    gw[k].push_back(make_uint4(g.x | g.y << 16, g.z | (IR + n) << 16, g.w, 0));
+                }
+            }
+        }
+        for (uint32_t k = 0; k < NW; ++k) {
+            catch_up(k, NL);
+            while (gw[k].empty() || gw[k].size() % 64) gw[k].resize(gw[k].size() + 32, make_uint4(0, 0, 0, 0));
+            D.gfirst[k + 1] = D.gfirst[k] + (uint32_t)(gw[k].size() / 32);
+            D.gdesc.insert(D.gdesc.end(), gw[k].begin(), gw[k].end());
+        }
+        for (uint32_t n = 0; n < N; ++n)
+            if (meta_op(D.desc[n].w) == OP_CONST) D.gconst.push_back(make_uint4(IR + n, const_value(D.desc[n]).x, const_value(D.desc[n]).y, 0));
+    }
     // Static fan-out cone estimate (reverse topological sum, capped): scheduling feature.
     D.cone.assign(n_net, 0.f);
     {
@@ -530,6 +599,9 @@ int upload_design(rtlfs_ctx *ctx, Design &D) {
     CU(D.d_rec.upload(D.rec));
     CU(D.d_net_static.upload(D.net_static));
     CU(D.d_chunks.upload(D.chunks));
+    CU(D.d_gdesc.upload(D.gdesc));
+    CU(D.d_gfirst.upload(D.gfirst));
+    CU(D.d_gconst.upload(D.gconst));
     CU(D.d_lvl_start.upload(D.lvl_start));
     CU(D.d_node_level.upload(D.node_level));
     CU(D.d_net_w.upload(D.net_w));
@@ -551,6 +623,7 @@ DevDesign dev_view(const Design &D) {
     v.T = D.T; v.n_fo = D.n_fo;
     v.n_chunks = (uint32_t)D.chunks.size();
     v.netinfo = D.d_netinfo.p; v.chunks = D.d_chunks.p;
+    v.gdesc = D.d_gdesc.p; v.gfirst = D.d_gfirst.p; v.gconst = D.d_gconst.p; v.n_gconst = (uint32_t)D.gconst.size();
     v.desc = D.d_desc.p; v.lvl_start = D.d_lvl_start.p; v.node_level = D.d_node_level.p;
     v.net_w = D.d_net_w.p; v.fo_off = D.d_fo_off.p; v.fo_idx = D.d_fo_idx.p; v.fo_lvl = D.d_fo_lvl.p; v.rec = D.d_rec.p; v.fo_edge = D.d_fo_edge.p;
     v.dreg_off = D.d_dreg_off.p; v.dreg_idx = D.d_dreg_idx.p; v.dreg_rec = D.d_dreg_rec.p; v.reg_d = D.d_reg_d.p;
@@ -561,73 +634,129 @@ DevDesign dev_view(const Design &D) {
 
 constexpr size_t SMEM_LIMIT = 227 * 1024;   // dynamic shared memory of one good-trace CTA
 
-// Cluster plan of a design for clusters of C CTAs: every level's nodes split into C
-// contiguous shares (CTA k owns its shares in level order, one value word per node),
-// registers split into C contiguous index blocks (their home CTAs), every operand
-// rewritten as the location of its value, and each CTA's chunk list (at least one chunk
-// per level, so every CTA joins every level's barrier).
+// Threads of a CTA of a cluster launch: at least eight warps, for the latch, and the one that
+// releases at the cluster's barrier.
+uint32_t cluster_threads(uint32_t width) { return std::max(width, 256u) + 32u; }
+
+// Words of a CTA that hold any plan of the design on clusters of C, with nodes and registers
+// evenly spread.
+uint64_t cluster_words(const Design &D, uint32_t C) {
+    return (D.N + C - 1) / C + 2ull * ((D.R + C - 1) / C) + D.I;
+}
+
+// Cluster plan of a design for clusters of C CTAs: each node's CTA and step, each register's home
+// CTA, every operand as the location of its value. List scheduling: nodes in level order, those
+// with the longest path behind them first, each go where they can be evaluated first -- the CTA of
+// an operand, or the least loaded one -- in the first step after their operands (two steps after
+// one of another CTA) in which that CTA has room. A third of the operands end up remote, where
+// an even split of each level left (C - 1) / C of them, at 2.5 cycles a lane.
 int build_cluster_plan(rtlfs_ctx *ctx, Design &D, uint32_t C, int lc) {
     auto P = std::make_unique<Design::ClusterPlan>();
     const uint32_t I = D.I, R = D.R, N = D.N, IR = I + R, NL = D.n_levels;
-    std::vector<uint32_t> own(C, 0), node_rank(N), node_slot(N);
-    std::vector<std::vector<uint4>> chunks(C);
-    for (uint32_t l = 0; l < NL; ++l) {
-        const uint32_t lo = D.lvl_start[l], n = D.lvl_start[l + 1] - lo;
-        for (uint32_t k = 0; k < C; ++k) {
-            const uint32_t a = lo + (uint32_t)((uint64_t)n * k / C);
-            const uint32_t b = lo + (uint32_t)((uint64_t)n * (k + 1) / C);
-            for (uint32_t x = a; x < b; ++x) { node_rank[x] = k; node_slot[x] = own[k] + (x - a); }
-            if (a == b) chunks[k].push_back(make_uint4(own[k], 0x80000000u, a, 0));
-            for (uint32_t x = a; x < b; x += GOOD_BLOCK) {
-                const uint32_t m = std::min(GOOD_BLOCK, b - x);
-                chunks[k].push_back(make_uint4(own[k] + (x - a), m | (x + m == b ? 0x80000000u : 0u), x, 0));
+    // words to spare in a CTA go to uneven shares
+    const uint64_t spare = SMEM_LIMIT / 8 - cluster_words(D, C);
+    const uint32_t n_even = (N + C - 1) / C, r_even = (R + C - 1) / C;
+    const uint32_t n_cap = (uint32_t)std::min<uint64_t>(n_even + spare / 2, 2ull * n_even);
+    const uint32_t r_cap = (uint32_t)std::min<uint64_t>(r_even + spare / 4, 2ull * r_even);
+    // nodes per step: a third above the mean of an even spread over the levels, 32 to 512
+    uint32_t width = 32;
+    while (width < GOOD_BLOCK && (uint64_t)width * C * NL < N + N / 3) width *= 2;
+    const uint32_t budget = NL + (NL + 19) / 20;   // steps a cycle should take
+
+    std::vector<uint32_t> height(N, 0), order(N);
+    for (uint32_t n = N; n-- > 0;) {
+        const uint4 s = good_slots(D.desc[n], IR + n);
+        for (uint32_t e : {s.x, s.y, s.z})
+            if (e >= IR && e != IR + n) height[e - IR] = std::max(height[e - IR], height[n] + 1);
+        order[n] = n;
+    }
+    std::stable_sort(order.begin(), order.end(), [&](uint32_t a, uint32_t b) {
+        return D.node_level[a] != D.node_level[b] ? D.node_level[a] < D.node_level[b] : height[a] > height[b];
+    });
+    std::vector<uint32_t> rank(N), step(N), slot(N), own(C, 0);
+    std::vector<std::vector<uint32_t>> used(C);   // nodes placed, per CTA and step
+    for (uint32_t n : order) {
+        const uint4 s = good_slots(D.desc[n], IR + n);
+        const uint32_t e[3] = {s.x, s.y, s.z};
+        uint32_t cand[4], nc = 0, bk = C, bs = 0;
+        uint64_t best = ~0ull;
+        for (uint32_t o : e)
+            if (o >= IR && o != IR + n && own[rank[o - IR]] < n_cap) cand[nc++] = rank[o - IR];
+        cand[nc++] = (uint32_t)(std::min_element(own.begin(), own.end()) - own.begin());
+        for (uint32_t c = 0; c < nc; ++c) {
+            const uint32_t k = cand[c];
+            uint32_t at = 0, remote = 0;
+            for (uint32_t o : e) {
+                if (o < IR || o == IR + n) continue;
+                const bool here = rank[o - IR] == k;
+                at = std::max(at, step[o - IR] + (here ? 1u : 2u));
+                remote += !here;
             }
-            own[k] += b - a;
+            while (at < used[k].size() && used[k][at] >= width) ++at;
+            const uint64_t late = at + height[n] > budget ? at + height[n] - budget : 0u, load = at < used[k].size() ? used[k][at] : 0u;
+            const uint64_t key = late << 40 | (uint64_t)remote << 36 | load << 24 | at;
+            if (key < best) { best = key; bk = k; bs = at; }
         }
+        rank[n] = bk;
+        step[n] = bs;
+        slot[n] = own[bk]++;
+        if (used[bk].size() <= bs) used[bk].resize(bs + 1, 0);
+        ++used[bk][bs];
+        P->steps = std::max(P->steps, bs + 1);
     }
-    std::vector<uint32_t> reg_off(C + 1), reg_home(R);
-    for (uint32_t k = 0; k <= C; ++k) reg_off[k] = (uint32_t)((uint64_t)R * k / C);
-    for (uint32_t k = 0; k < C; ++k)
-        for (uint32_t r = reg_off[k]; r < reg_off[k + 1]; ++r) reg_home[r] = k;
+    P->steps += P->steps % 2;
+    P->width = width;
     P->own = *std::max_element(own.begin(), own.end());
-    P->rown = 0;
-    for (uint32_t k = 0; k < C; ++k) P->rown = std::max(P->rown, reg_off[k + 1] - reg_off[k]);
-    if ((uint64_t)P->own + 2ull * P->rown + I > CL_WORD) return fail(ctx, RTLFS_E_ARG, "design too large for a cluster plan");
-    auto loc = [&](uint32_t net) -> uint32_t {
-        if (net < I) return CL_SELF | (P->own + 2 * P->rown + net);
-        if (net < IR) {
-            const uint32_t r = net - I, k = reg_home[r];
-            return CL_REG | (k << CL_RANK_SHIFT) | (P->own + r - reg_off[k]);
+    // a register's home: the CTA of its D node, else (or when that is full) the emptiest
+    std::vector<uint32_t> reg_n(C, 0), reg_home(R), reg_at(R);
+    for (uint32_t r = 0; r < R; ++r) {
+        const uint32_t d = D.reg_d[r];
+        uint32_t k = d >= IR ? rank[d - IR] : C;
+        if (k == C || reg_n[k] >= r_cap) {
+            const uint32_t m = (uint32_t)(std::min_element(reg_n.begin(), reg_n.end()) - reg_n.begin());
+            if (k != C) P->latch_sync = 1;
+            k = m;
         }
-        const uint32_t x = net - IR;
-        return (node_rank[x] << CL_RANK_SHIFT) | node_slot[x];
+        reg_home[r] = k;
+        reg_at[r] = reg_n[k]++;
+    }
+    P->rown = *std::max_element(reg_n.begin(), reg_n.end());
+    auto loc = [&](uint32_t net, uint32_t me) -> uint32_t {
+        if (net < I) return CL_SELF | (P->own + 2 * P->rown + net);
+        const bool reg = net < IR;
+        const uint32_t k = reg ? reg_home[net - I] : rank[net - IR];
+        return (reg ? CL_REG : 0u) | (k == me ? CL_SELF : 0u) | (k << CL_RANK_SHIFT) | (reg ? P->own + reg_at[net - I] : slot[net - IR]);
     };
-    std::vector<uint4> cdesc((size_t)C * P->own, make_uint4(0, 0, 0, 0));
-    for (uint32_t x = 0; x < N; ++x) {
-        uint4 d = D.desc[x];
-        const int no = n_ops(meta_op(d.w));
-        if (no >= 1) d.x = loc(d.x);
-        if (no >= 2) d.y = loc(d.y);
-        if (no >= 3) d.z = loc(d.z);
-        cdesc[(size_t)node_rank[x] * P->own + node_slot[x]] = d;
+    const size_t per_cta = (size_t)P->steps * width;
+    std::vector<uint4> cdesc(C * per_cta + 1, make_uint4(0, 0, 0, 0));
+    std::vector<std::vector<uint4>> consts(C);
+    for (auto &u : used) std::fill(u.begin(), u.end(), 0u);
+    for (uint32_t n = 0; n < N; ++n) {   // in node order within a step: neighbours share trace lines
+        const uint32_t k = rank[n];
+        const uint4 s = good_slots(D.desc[n], IR + n);
+        cdesc[k * per_cta + (size_t)step[n] * width + used[k][step[n]]++] =
+            make_uint4(loc(s.x, k) | n << CL_BITS, loc(s.y, k) | n >> (32 - CL_BITS) << CL_BITS, loc(s.z, k) | slot[n] << CL_BITS,
+                       s.w | slot[n] >> (32 - CL_BITS) << CL_SLOT_HI);
+        if (meta_op(D.desc[n].w) == OP_CONST) {
+            const uint2 v = const_value(D.desc[n]);
+            consts[k].push_back(make_uint4(slot[n], v.x, v.y, 0));
+        }
     }
-    std::vector<uint4> creg(R);
-    for (uint32_t r = 0; r < R; ++r) creg[r] = make_uint4(r, loc(D.reg_d[r]), D.net_w[I + r], D.reg_d[r]);
-    std::vector<uint4> call;
-    std::vector<uint32_t> ch_off(C + 1, 0);
-    P->max_ch = 0;
+    std::vector<uint4> ccall, creg(R);
+    std::vector<uint32_t> const_off(C + 1, 0), reg_off(C + 1, 0);
     for (uint32_t k = 0; k < C; ++k) {
-        ch_off[k] = (uint32_t)call.size();
-        call.insert(call.end(), chunks[k].begin(), chunks[k].end());
-        P->max_ch = std::max<uint32_t>(P->max_ch, (uint32_t)chunks[k].size());
+        ccall.insert(ccall.end(), consts[k].begin(), consts[k].end());
+        const_off[k + 1] = (uint32_t)ccall.size();
+        reg_off[k + 1] = reg_off[k] + reg_n[k];
     }
-    ch_off[C] = (uint32_t)call.size();
-    P->smem = good_cluster_smem_bytes(P->own, P->rown, I, P->max_ch);
+    for (uint32_t r = 0; r < R; ++r)
+        creg[reg_off[reg_home[r]] + reg_at[r]] = make_uint4(r, loc(D.reg_d[r], reg_home[r]), D.net_w[I + r], D.reg_d[r]);
+    P->smem = good_cluster_smem_bytes(P->own, P->rown, I);
     CU(P->d_desc.upload(cdesc));
-    CU(P->d_chunk.upload(call));
     CU(P->d_reg.upload(creg));
-    CU(P->d_ch_off.upload(ch_off));
     CU(P->d_reg_off.upload(reg_off));
+    CU(P->d_const.upload(ccall));
+    CU(P->d_const_off.upload(const_off));
     D.plan[lc] = std::move(P);
     return RTLFS_OK;
 }
@@ -635,21 +764,21 @@ int build_cluster_plan(rtlfs_ctx *ctx, Design &D, uint32_t C, int lc) {
 // Whether clusters of C CTAs can run design D's good trace; builds the plan on first use.
 int cluster_usable(rtlfs_ctx *ctx, Design &D, uint32_t C, int lc, bool *ok) {
     *ok = false;
+    if (cluster_words(D, C) * 8 > SMEM_LIMIT || D.N >= 1u << 22) return RTLFS_OK;
     if (!D.plan[lc]) {
         int rc = build_cluster_plan(ctx, D, C, lc);
         if (rc != RTLFS_OK) return rc;
     }
     Design::ClusterPlan &P = *D.plan[lc];
     if (P.smem > SMEM_LIMIT) return RTLFS_OK;
-    if ((uint64_t)D.T * P.max_ch >= (1ull << 32)) return RTLFS_OK;
-    if (P.usable < 0) P.usable = good_cluster_max_active(C, P.smem) > 0 ? 1 : 0;
+    if (P.usable < 0) P.usable = good_cluster_max_active(C, cluster_threads(P.width), P.smem) > 0 ? 1 : 0;
     *ok = P.usable == 1;
     return RTLFS_OK;
 }
 
 // Allocate traces, choose each design's good-trace form and upload the design table and
 // the launch lists: one CTA with net values in shared memory when the design fits, else
-// the smallest cluster whose CTAs hold the design in distributed shared memory, else one
+// a cluster whose CTAs hold the design in distributed shared memory, else one
 // CTA with net values in the global trace. ctx->good_cluster overrides the choice:
 // 1 = one CTA, 2..16 = clusters of that size.
 int prepare_good(rtlfs_ctx *ctx) {
@@ -657,6 +786,13 @@ int prepare_good(rtlfs_ctx *ctx) {
     std::vector<uint32_t> l_smem, l_glob, l_cl[5];
     GoodLaunch g{};
     const uint32_t force = ctx->good_cluster;
+    // Larger clusters are faster (48k nodes: 44.5, 34.4, 28.8, 28.2 us a cycle on 2, 4, 8, 16), but
+    // the designs' clusters together should stay within the SMs that a campaign leaves to them.
+    uint32_t n_big = 0;
+    for (const Design *D : ctx->designs)
+        n_big += good_smem_bytes(true, D->n_net, D->R, (uint32_t)D->chunks.size(), ctx->good_staging != 0) > SMEM_LIMIT;
+    int lc_want = 4;
+    while (lc_want > 1 && (n_big << lc_want) > (uint32_t)ctx->n_sm / 4) --lc_want;
     for (size_t i = 0; i < ctx->designs.size(); ++i) {
         Design &D = *ctx->designs[i];
         const size_t cells = (size_t)D.n_net * D.T;
@@ -682,13 +818,13 @@ int prepare_good(rtlfs_ctx *ctx) {
                 g.max_net_s = mn; g.max_reg_s = mr; g.max_ch_s = mc;
             } else {
                 if (force == 0) {
-                    for (lc = 1; (1u << lc) <= CL_MAX; ++lc) {
-                        bool ok = false;
+                    bool ok = false;   // the size wanted, else the next larger, else a smaller one
+                    for (int k = 0; k < 4 && !ok; ++k) {
+                        lc = lc_want + k <= 4 ? lc_want + k : 4 - k;
                         int rc = cluster_usable(ctx, D, 1u << lc, lc, &ok);
                         if (rc != RTLFS_OK) return rc;
-                        if (ok) break;
                     }
-                    if ((1u << lc) > CL_MAX) lc = 0;
+                    if (!ok) lc = 0;
                 }
                 if (lc == 0) {
                     l_glob.push_back((uint32_t)i);
@@ -699,10 +835,12 @@ int prepare_good(rtlfs_ctx *ctx) {
         if (lc > 0) {
             const Design::ClusterPlan &P = *D.plan[lc];
             v.cl_own = P.own; v.cl_rown = P.rown;
-            v.cl_desc = P.d_desc.p; v.cl_chunk = P.d_chunk.p; v.cl_ch_off = P.d_ch_off.p;
+            v.cl_steps = P.steps; v.cl_width = P.width; v.cl_latch_sync = P.latch_sync; v.cl_desc = P.d_desc.p;
             v.cl_reg = P.d_reg.p; v.cl_reg_off = P.d_reg_off.p;
+            v.cl_const = P.d_const.p; v.cl_const_off = P.d_const_off.p;
             l_cl[lc].push_back((uint32_t)i);
             g.smem_cl[lc] = std::max(g.smem_cl[lc], P.smem);
+            g.thr_cl[lc] = std::max(g.thr_cl[lc], cluster_threads(P.width));
         }
         tab.push_back(v);
     }
@@ -753,7 +891,7 @@ int launch_good_lists(rtlfs_ctx *ctx, cudaStream_t stream, uint32_t t0, uint32_t
     for (int lc = 1; lc < 5; ++lc) {
         if (!g.n_cl[lc]) continue;
         if (int r = next_stream(&st)) return r;
-        CU(launch_good_cluster(ctx->d_designs.p, ctx->d_list_cl[lc].p, g.n_cl[lc], 1u << lc, g.smem_cl[lc], ctx->d_err.p,
+        CU(launch_good_cluster(ctx->d_designs.p, ctx->d_list_cl[lc].p, g.n_cl[lc], 1u << lc, g.thr_cl[lc], g.smem_cl[lc], ctx->d_err.p,
                                st, t0, t1));
     }
     for (int j = 1; j < k; ++j) {   // join

@@ -42,6 +42,13 @@ struct DevDesign {
     uint32_t n_chunks;          // good-trace chunks (<= GOOD_BLOCK nodes each, never across levels)
     const uint4    *netinfo;    // [n_net]
     const uint2    *chunks;     // [n_chunks] {first node, end node | 1<<31 if last of its level}
+    // Good trace with net values in shared memory: each warp's groups of 32 nodes, an even number
+    // of them, none for a design of more than 65535 nets.
+    const uint4    *gdesc;      // [groups][32] {slot 0 net | slot 1 net << 16, select | own net << 16, GM_*,
+                                // levels that end after the group}
+    const uint32_t *gfirst;     // [GOOD_BLOCK / 32 + 1] first group of each warp
+    const uint4    *gconst;     // [n_gconst] constant nodes: {net, value lo, hi, 0}
+    uint32_t n_gconst;
     const uint4    *desc;       // [N]
     const uint32_t *lvl_start;  // [n_levels + 1] node-index range of each level
     const uint16_t *node_level; // [N]
@@ -66,28 +73,42 @@ struct DevDesign {
     uint64_t *rows;             // [T][n_net] good trace, one row per cycle
     uint64_t *gcol;             // [n_net][T] good trace, one column per net
     // Cluster good trace (designs too large for one CTA's shared memory): the layout of
-    // one CTA's value area and each CTA's descriptor, chunk and register lists.
+    // one CTA's value area, its schedule and its register and constant lists.
     uint32_t cl_own;            // node values per CTA (words)
     uint32_t cl_rown;           // registers per CTA (words per bank)
-    const uint4    *cl_desc;    // [C][cl_own] descriptors, operands as cluster locations
-    const uint4    *cl_chunk;   // chunk lists {first slot, count | 1<<31 at a level's end, first node, 0}
-    const uint32_t *cl_ch_off;  // [C + 1] chunk list of each CTA
+    uint32_t cl_steps;          // steps of a cycle, an even number
+    uint32_t cl_width;          // nodes a CTA evaluates per step, at most (a multiple of 32)
+    uint32_t cl_latch_sync;     // some register's D net is a node of another CTA
+    const uint4    *cl_desc;    // [C][cl_steps][cl_width] records, and a blank one
     const uint4    *cl_reg;     // {register, D location, width, D net} by home CTA
-    const uint32_t *cl_reg_off; // [C + 1] registers of each CTA (a contiguous index range)
+    const uint32_t *cl_reg_off; // [C + 1] registers of each CTA
+    const uint4    *cl_const;   // {slot, value lo, hi, 0}: constant nodes by CTA
+    const uint32_t *cl_const_off; // [C + 1]
 };
+
+// A node of the good trace (good_eval): value slots 0 and 1 hold operands a and b, or b and c of
+// a MUX2, whose a is the select. Byte 0: shift amount k, byte 1: 64 - width; the top bits of the
+// four bytes select the terms of the bitwise result. A constant reads its own net, set up once.
+constexpr uint32_t GM_A = 1u << 7, GM_B = 1u << 15, GM_C = 1u << 23, GM_D = 1u << 31;
+constexpr uint32_t GM_LEFT = 1u << 16, GM_SUM = 1u << 17, GM_CMP = 1u << 18, GM_EQ = 1u << 19;
+constexpr uint32_t GM_NEG = 1u << 20, GM_MUX = 1u << 21, GM_LAST = 1u << 24, GM_VALID = 1u << 25;
 
 // Evaluation masks of a packed record's meta (pack_eval).
 constexpr uint32_t PM_LEFT = 1u << 24, PM_SUM = 1u << 25, PM_CMP = 1u << 26;
 constexpr uint32_t PM_A = 1u << 28, PM_B = 1u << 29, PM_C = 1u << 30, PM_D = 1u << 31;
 
-// A net's location for the cluster good trace, 32 bits: the word in the holding CTA's
-// value area (node values [0, own), register banks [own, own + 2 rown), inputs after
-// them), the holder's rank in the cluster, and two flags: a register (add the bank of
-// the cycle's parity) and an input (every CTA holds a copy: read the local one).
-constexpr uint32_t CL_WORD = 0x00FFFFFFu;
-constexpr uint32_t CL_RANK_SHIFT = 24;
-constexpr uint32_t CL_REG = 1u << 28;
-constexpr uint32_t CL_SELF = 1u << 29;
+// A net's location for the cluster good trace, 21 bits: the word in the holding CTA's value area
+// (node values [0, own), register banks [own, own + 2 rown), inputs after them), the holder's
+// rank in the cluster, and two flags: a register (add the bank of the cycle's parity) and a value
+// the reading CTA holds itself (its own nodes and registers, and the inputs, of which every CTA
+// holds a copy). A node's record: the locations of value slots 0 and 1 and of the select in the
+// low bits of x, y, z; w = GM_*; its number in the design in the upper bits of x and y (11 + 11)
+// and its own word in those of z and w (11, then 4 from bit CL_SLOT_HI).
+constexpr uint32_t CL_WORD = 0x7FFFu;
+constexpr uint32_t CL_RANK_SHIFT = 15;
+constexpr uint32_t CL_REG = 1u << 19;
+constexpr uint32_t CL_SELF = 1u << 20;
+constexpr uint32_t CL_BITS = 21, CL_SLOT_HI = 26;
 constexpr uint32_t CL_MAX = 16;   // largest cluster (non-portable size on sm_103a)
 
 // All faults of all designs, concatenated in design order.
@@ -318,13 +339,13 @@ cudaError_t launch_heavy_window(const DevDesign *d_designs, DevFaults f, WinHeav
 cudaError_t launch_transpose(uint64_t *gcol, const uint64_t *rows, uint32_t n_net, uint32_t T,
                              cudaStream_t stream);
 // Shared memory of one cluster good-trace CTA for a design's layout.
-size_t good_cluster_smem_bytes(uint32_t own, uint32_t rown, uint32_t n_inputs, uint32_t max_chunks);
-// Clusters of C CTAs with `smem` bytes each that can be resident at once (0: none).
-int good_cluster_max_active(uint32_t C, size_t smem);
+size_t good_cluster_smem_bytes(uint32_t own, uint32_t rown, uint32_t n_inputs);
+// Clusters of C CTAs with that many threads and `smem` bytes each that can be resident at once (0: none).
+int good_cluster_max_active(uint32_t C, uint32_t threads, size_t smem);
 // Good trace of the listed designs over cycles [t_begin, t_end), one cluster of C CTAs each.
 // A launch that does not run in clusters of C CTAs does nothing and sets bit 2 of *err.
 cudaError_t launch_good_cluster(const DevDesign *d_designs, const uint32_t *design_list,
-                                uint32_t n_list, uint32_t C, size_t smem, uint32_t *err,
+                                uint32_t n_list, uint32_t C, uint32_t threads, size_t smem, uint32_t *err,
                                 cudaStream_t stream, uint32_t t_begin, uint32_t t_end);
 cudaError_t launch_light(const DevDesign *d_designs, DevFaults f, Queues q, int cap, int block,
                          int grid, cudaStream_t stream);

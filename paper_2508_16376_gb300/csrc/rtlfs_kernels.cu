@@ -27,48 +27,166 @@ namespace rtlfs {
 // ===================================================================================
 // Good-machine trace. One CTA per design walks the cycles; inside a cycle the nodes of
 // one topological level are independent and are spread over the threads, with a
-// barrier between levels. The node list is cut into chunks of at most GOOD_BLOCK nodes
-// that never straddle a level, so every thread owns at most one node per chunk. Each
-// thread loads its node descriptors two chunks ahead of use (wrapping into the next
-// cycle), so no evaluation waits on a global load. Net values of the current cycle live
-// in shared memory when they fit (USE_SMEM) and are streamed to the row-major trace
-// rows[t][net].
+// barrier between levels. Net values of the current cycle live in shared memory when they
+// fit (good_trace_smem_kernel) and are streamed to the row-major trace rows[t][net]; else
+// the trace itself holds them (good_trace_kernel).
+// What bounds it is the serial chain of a level: an operand read, one evaluation, a write and
+// the CTA's barrier (115 cycles without the evaluation), and for wide levels the issue of
+// some 87 instructions per 32 nodes and 6 bank passes per operand read. So a warp walks its
+// own list of 32-node groups, whose records hold all a group needs and say how many levels
+// end after it: a warp without nodes in a level only meets the barrier, and no chunk table,
+// bound check or select stands between two barriers. 20k nodes on 46 levels: 27.8 us a cycle
+// with a chunk table and a switch over the ops, 19.7 with good_eval, 15.3 with the lists.
 // ===================================================================================
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
-template <bool USE_SMEM>
+// One node of the good machine: every op's result from the same straight line of code. A warp
+// holds nodes of many ops, and a switch ran each op's case in turn, with a branch and a
+// reconvergence each: 1150 of a level's cycles.
+__device__ __forceinline__ uint64_t good_eval(uint32_t w, uint64_t x, uint64_t y, uint64_t s) {
+    if (s) y = x;              // MUX2: slot 0 instead of slot 1
+    uint64_t xl, xr;           // shifts by 64 give 0
+    asm("shl.b64 %0, %1, %2;" : "=l"(xl) : "l"(x), "r"(w & 127u));
+    asm("shr.u64 %0, %1, %2;" : "=l"(xr) : "l"(x), "r"(w & 127u));
+    const uint64_t xs = w & GM_LEFT ? xl : xr;
+    uint32_t ma, mb, mc, md;   // the top bit of each byte, spread over a word
+    asm("prmt.b32 %0, %1, 0, 0x8888;" : "=r"(ma) : "r"(w));
+    asm("prmt.b32 %0, %1, 0, 0x9999;" : "=r"(mb) : "r"(w));
+    asm("prmt.b32 %0, %1, 0, 0xaaaa;" : "=r"(mc) : "r"(w));
+    asm("prmt.b32 %0, %1, 0, 0xbbbb;" : "=r"(md) : "r"(w));
+    auto bits = [&](uint32_t p, uint32_t q) { return (p & q & ma) ^ (p & mb) ^ (q & mc) ^ md; };
+    uint32_t lo = bits((uint32_t)xs, (uint32_t)y), hi = bits((uint32_t)(xs >> 32), (uint32_t)(y >> 32));
+    // x + y, or x - y = x + ~y + 1, whose carry says x >= y
+    const uint32_t ng = w & GM_NEG ? ~0u : 0u;
+    uint32_t sl, sh, cy;
+    asm("{\n\t.reg .u32 t;\n\t"
+        "add.cc.u32 t, %7, 1;\n\t"
+        "addc.cc.u32 %0, %3, %5;\n\t"
+        "addc.cc.u32 %1, %4, %6;\n\t"
+        "addc.u32 %2, 0, 0;\n\t}"
+        : "=&r"(sl), "=&r"(sh), "=r"(cy)
+        : "r"((uint32_t)x), "r"((uint32_t)(x >> 32)), "r"((uint32_t)y ^ ng), "r"((uint32_t)(y >> 32) ^ ng), "r"(ng));
+    if (w & GM_SUM) { lo = sl; hi = sh; }
+    const bool cmp = w & GM_EQ ? (sl | sh) == 0u : cy == 0u;
+    if (w & GM_CMP) { lo = cmp ? 1u : 0u; hi = 0u; }
+    return ((uint64_t)hi << 32 | lo) & (~0ull >> ((w >> 8) & 63u));
+}
+
+template <int KR>
 __global__ void __launch_bounds__(GOOD_BLOCK, 1)
-good_trace_kernel(const DevDesign *__restrict__ designs, const uint32_t *__restrict__ list,
-                  uint32_t max_net, uint32_t max_reg, uint32_t max_chunks, uint32_t t_begin, uint32_t t_end) {
+good_trace_smem_kernel(const DevDesign *__restrict__ designs, const uint32_t *__restrict__ list,
+                       uint32_t max_net, uint32_t t_begin, uint32_t t_end) {
     extern __shared__ __align__(128) uint64_t gsm[];
     const DevDesign &D = designs[list[blockIdx.x]];
-    const uint32_t I = D.I, R = D.R, IR = I + R, n_net = D.n_net, NC = D.n_chunks;
+    const uint32_t I = D.I, R = D.R, n_net = D.n_net;
+    const uint32_t T = min(D.T, t_end);   // last cycle (exclusive) of this launch
+    if (t_begin >= T) return;
+    const uint32_t tid = threadIdx.x, B = GOOD_BLOCK;
+    uint64_t *const val = gsm;              // [max_net]
+    uint64_t *const qn = gsm + max_net;     // [R]: used beyond the first KR registers of each thread
+    const uint32_t g_begin = D.gfirst[tid >> 5], g_end = D.gfirst[(tid >> 5) + 1];   // this warp's groups
+    const uint4 *__restrict__ const gd = D.gdesc + (size_t)g_begin * 32 + (tid & 31u);
+    const uint64_t *__restrict__ stim = D.stim;
+    uint64_t *__restrict__ const rows = D.rows;
+    for (uint32_t k = tid; k < D.n_gconst; k += B) {
+        const uint4 g = D.gconst[k];
+        val[g.x] = (uint64_t)g.z << 32 | g.y;
+    }
+    // this thread's input and its first registers, kept in registers for every cycle
+    const uint64_t in_mask = tid < I ? wmask(D.net_w[tid]) : 0ull;
+    uint32_t rd[KR], rw[KR];
+    uint64_t q[KR];
+    const uint64_t *prev = rows + (size_t)(t_begin ? t_begin - 1 : 0) * n_net;   // resume: its row
+#pragma unroll
+    for (int k = 0; k < KR; ++k) {
+        const uint32_t r = tid + k * B;
+        rd[k] = r < R ? D.reg_d[r] : 0u;
+        rw[k] = r < R ? 64u - D.net_w[I + r] : 0u;
+        q[k] = r < R && t_begin ? prev[rd[k]] & (~0ull >> rw[k]) : 0ull;
+    }
+    for (uint32_t r = tid + KR * B; r < R; r += B) qn[r] = t_begin ? prev[D.reg_d[r]] & wmask(D.net_w[I + r]) : 0ull;
+
+    // Records two groups ahead in registers (wrapping into the next cycle). The load has no
+    // condition: merging it with another value would wait for it at once.
+    const uint32_t END = (g_end - g_begin) * 32;
+    uint32_t off = 0;
+    auto prefetch = [&]() -> uint4 {
+        const uint4 d = __ldg(gd + off);
+        off = off + 32 == END ? 0u : off + 32;
+        return d;
+    };
+    uint4 d0 = prefetch(), d1 = prefetch();
+    uint64_t s_next = tid < I ? __ldg(stim + (size_t)t_begin * I + tid) : 0ull;
+
+    for (uint32_t t = t_begin; t < T; ++t) {
+        uint64_t *__restrict__ const row = rows + (size_t)t * n_net;
+        const uint64_t s_cur = s_next & in_mask;
+        if (tid < I) {
+            if (t + 1 < T) s_next = __ldg(stim + (size_t)(t + 1) * I + tid);
+            val[tid] = s_cur;
+            row[tid] = s_cur;
+        }
+        for (uint32_t i = tid + B; i < I; i += B) {
+            const uint64_t v = __ldg(stim + (size_t)t * I + i) & wmask(D.net_w[i]);
+            val[i] = v;
+            row[i] = v;
+        }
+#pragma unroll
+        for (int k = 0; k < KR; ++k) {
+            const uint32_t r = tid + k * B;
+            if (r < R) {
+                val[I + r] = q[k];
+                row[I + r] = q[k];
+            }
+        }
+        for (uint32_t r = tid + KR * B; r < R; r += B) {
+            val[I + r] = qn[r];
+            row[I + r] = qn[r];
+        }
+        __syncthreads();
+        auto group = [&](uint4 &d) {
+            const uint32_t in = d.x, sd = d.y, w = d.z, nb = d.w;
+            d = prefetch();
+            if (w & GM_VALID) {
+                const uint64_t x = val[in & 0xFFFFu], y = val[in >> 16];
+                uint64_t s = 0ull;
+                if (w & GM_MUX) s = val[sd & 0xFFFFu];
+                const uint64_t v = good_eval(w, x, y, s);
+                val[sd >> 16] = v;
+                row[sd >> 16] = v;
+            }
+            if (nb) __syncthreads();   // a level is complete
+#pragma unroll 1
+            for (uint32_t k = 1; k < nb; ++k) __syncthreads();
+        };
+#pragma unroll 1
+        for (uint32_t g = g_begin; g < g_end; g += 2) {
+            group(d0);
+            group(d1);
+        }
+#pragma unroll
+        for (int k = 0; k < KR; ++k)
+            if (tid + k * B < R) q[k] = val[rd[k]] & (~0ull >> rw[k]);
+        for (uint32_t r = tid + KR * B; r < R; r += B) qn[r] = val[D.reg_d[r]] & wmask(D.net_w[I + r]);
+        __syncthreads();
+    }
+}
+
+// The same walk for a design whose values do not fit in shared memory (and is kept on one CTA):
+// operands are read back from the trace row.
+__global__ void __launch_bounds__(GOOD_BLOCK, 1)
+good_trace_kernel(const DevDesign *__restrict__ designs, const uint32_t *__restrict__ list, uint32_t t_begin, uint32_t t_end) {
+    extern __shared__ __align__(128) uint64_t gsm[];
+    const DevDesign &D = designs[list[blockIdx.x]];
+    const uint32_t I = D.I, IR = I + D.R, n_net = D.n_net, NC = D.n_chunks;
     const uint32_t T = min(D.T, t_end);   // last cycle (exclusive) of this launch
     if (t_begin >= T) return;
     const uint32_t tid = threadIdx.x, B = blockDim.x;
-    const size_t vwords = USE_SMEM ? (size_t)max_net + max_reg : 0;   // u64 words of values
-    uint64_t *val = gsm;                                     // [max_net] when USE_SMEM
-    uint64_t *qn = gsm + (USE_SMEM ? max_net : 0);           // [max_reg] when USE_SMEM
-    uint2 *ch = reinterpret_cast<uint2 *>(gsm + vwords);     // [max_chunks]
-    (void)max_chunks;
+    uint2 *ch = reinterpret_cast<uint2 *>(gsm);     // [NC]
     for (uint32_t c = tid; c < NC; c += B) ch[c] = D.chunks[c];
-    // this thread's input and its first two registers, kept in registers for every cycle
-    const uint64_t in_mask = tid < I ? wmask(D.net_w[tid]) : 0ull;
-    const uint32_t r0 = tid, r1 = tid + B;
-    const uint32_t rd0 = r0 < R ? D.reg_d[r0] : 0, rd1 = r1 < R ? D.reg_d[r1] : 0;
-    const uint64_t rm0 = r0 < R ? wmask(D.net_w[I + r0]) : 0, rm1 = r1 < R ? wmask(D.net_w[I + r1]) : 0;
-    if (USE_SMEM && t_begin > 0) {   // resume: register values of t_begin from row t_begin-1
-        const uint64_t *prev = D.rows + (size_t)(t_begin - 1) * n_net;
-        for (uint32_t r = tid; r < R; r += B) qn[r] = prev[D.reg_d[r]] & wmask(D.net_w[I + r]);
-    }
     __syncthreads();
-
-    // Each thread prefetches its node descriptor two chunks ahead into registers (coalesced
-    // loads from the L2-resident op graph, wrapping into the next cycle), so no evaluation
-    // waits on a global load; chunks of one level are independent, so only a chunk that
-    // ends a level is followed by a barrier.
     uint32_t cf = 0;                           // chunk of the next prefetch (wraps)
     auto prefetch = [&]() -> uint4 {
         if (NC == 0) return make_uint4(0u, 0u, 0u, 0u);   // a design without nodes
@@ -79,19 +197,13 @@ good_trace_kernel(const DevDesign *__restrict__ designs, const uint32_t *__restr
     };
     uint4 dq0 = prefetch();
     uint4 dq1 = prefetch();
-    uint64_t s_next = (tid < I) ? __ldg(D.stim + (size_t)t_begin * I + tid) : 0ull;
-
     for (uint32_t t = t_begin; t < T; ++t) {
         uint64_t *row = D.rows + (size_t)t * n_net;
-        const uint64_t s_cur = s_next;
-        if (tid < I && t + 1 < T) s_next = __ldg(D.stim + (size_t)(t + 1) * I + tid);
         for (uint32_t i = tid; i < IR; i += B) {
             uint64_t v;
-            if (i < I) v = (i == tid ? s_cur : __ldg(D.stim + (size_t)t * I + i)) & (i == tid ? in_mask : wmask(D.net_w[i]));
+            if (i < I) v = __ldg(D.stim + (size_t)t * I + i) & wmask(D.net_w[i]);
             else if (t == 0) v = 0ull;
-            else if (USE_SMEM) v = qn[i - I];
             else v = (row - n_net)[D.reg_d[i - I]] & wmask(D.net_w[i]);   // previous row
-            if (USE_SMEM) val[i] = v;
             row[i] = v;
         }
         __syncthreads();
@@ -102,27 +214,20 @@ good_trace_kernel(const DevDesign *__restrict__ designs, const uint32_t *__restr
             dq0 = dq1;
             dq1 = prefetch();
             if (n < (b.y & 0x7FFFFFFFu)) {
-                const uint32_t op = meta_op(d0.w);
-                const int no = n_operands(op);
+                const int no = n_operands(meta_op(d0.w));
                 uint64_t a = 0, bb = 0, cc = 0;
-                if (no >= 1) a = USE_SMEM ? val[d0.x] : row[d0.x];
-                if (no >= 2) bb = USE_SMEM ? val[d0.y] : row[d0.y];
-                if (no >= 3) cc = USE_SMEM ? val[d0.z] : row[d0.z];
-                const uint64_t v = eval_op(d0, a, bb, cc);
-                if (USE_SMEM) val[IR + n] = v;
-                row[IR + n] = v;
+                if (no >= 1) a = row[d0.x];
+                if (no >= 2) bb = row[d0.y];
+                if (no >= 3) cc = row[d0.z];
+                row[IR + n] = eval_op(d0, a, bb, cc);
             }
             if (b.y & 0x80000000u) __syncthreads();   // the level's values are complete
-        }
-        if (USE_SMEM) {
-            if (r0 < R) qn[r0] = val[rd0] & rm0;
-            if (r1 < R) qn[r1] = val[rd1] & rm1;
-            for (uint32_t r = tid + 2 * B; r < R; r += B) qn[r] = val[D.reg_d[r]] & wmask(D.net_w[I + r]);
         }
         __syncthreads();
     }
 }
 
+// ===================================================================================
 // Staged form of the single-CTA good trace: GOOD_BLOCK consumer threads plus one producer
 // warp. The producer copies each chunk's descriptors into a ring of GOOD_NSTAGE shared
 // buffers with bulk asynchronous copies (completion counted in bytes on the buffer's "full"
@@ -297,18 +402,24 @@ good_trace_staged_kernel(const DevDesign *__restrict__ designs, const uint32_t *
 
 // ===================================================================================
 // Good-machine trace of a design too large for one CTA's shared memory: one cluster of
-// C CTAs (2..16) per design. Each CTA owns a contiguous share of every level's nodes and
-// keeps their values of the current cycle in its own shared memory; a node reads each
-// operand where it lives through distributed shared memory (mapa + ld.shared::cluster),
-// its descriptor carrying the operand's location (CL_*). A register lives in its home
-// CTA in two banks selected by the cycle's parity: the latch of cycle t fills bank
-// (t+1)&1 while other registers' latches may still read Q_t from bank t&1 (a register
-// fed by a register). Every CTA keeps its own copy of the inputs. A cluster barrier
-// (release/acquire, so a level's values are visible cluster-wide) ends every level and
-// the latch. Each CTA prefetches its own descriptor list three chunks ahead into
-// registers (one more than the single-CTA kernel: a remote operand read and the cluster
-// barrier make a level longer); a level in which a CTA owns no node is an empty chunk
-// that only joins the barrier.
+// C CTAs (2..16) per design. A schedule made when the design is planned gives each node a CTA,
+// which keeps the node's value of the current cycle in its shared memory, and a step. A
+// node reads each operand where it lives; one of another CTA comes through distributed shared
+// memory (mapa + ld.shared::cluster). A node's step lies after those of its operands in the
+// same CTA, whose threads meet at a CTA barrier after every step, and at least two steps
+// after those of its operands elsewhere: every thread arrives on the cluster's barrier
+// (release) after a step and waits for that arrival's phase (acquire) after the next, so the
+// barrier's latency passes under a step's work and a node's nearest operand is local. The last
+// warp releases for its CTA: a release waits for its own thread's loads and stores in flight
+// and for some 300 cycles more, so it does nothing else during the steps and fences before it
+// waits. What bounds it is a step's chain of fence, barrier (400 cycles) and remote read (250,
+// and 2.5 a lane). 48k nodes on 44 levels: 78.8 us a cycle on 2 CTAs with levels split evenly and
+// a barrier each, 28.2 on 16 with the schedule; 200k nodes on 72 levels, 16 CTAs: 113 and 54.
+// A register lives in its home CTA (its D net's, where possible) in two banks selected by the
+// cycle's parity: the latch of cycle t fills bank (t+1)&1 while other registers' latches may
+// still read Q_t from bank t&1 (a register fed by a register). Every CTA keeps its own copy of
+// the inputs. A cluster barrier ends the latch, so nothing of a cycle is overwritten while
+// another CTA may read it.
 // ===================================================================================
 __device__ __forceinline__ uint32_t cluster_rank() {
     uint32_t r;
@@ -327,16 +438,24 @@ __device__ __forceinline__ void cluster_sync() {
                  "barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// 64-bit load from the same shared-memory offset in CTA `rank` of this cluster.
-__device__ __forceinline__ uint64_t dsm_load(uint32_t local_addr, uint32_t rank) {
-    uint32_t ra;
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+// 64-bit load from a shared-memory address of this CTA (self != 0), or from the same address in
+// CTA `rank` of the cluster, without a branch.
+__device__ __forceinline__ uint64_t dsm_load(uint32_t addr, uint32_t rank, uint32_t self) {
     uint64_t v;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(local_addr), "r"(rank));
-    asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(ra));
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .u32 ra;\n\t"
+                 "setp.ne.u32 p, %3, 0;\n\t"
+                 "mapa.shared::cluster.u32 ra, %1, %2;\n\t"
+                 "@p ld.shared.u64 %0, [%1];\n\t"
+                 "@!p ld.shared::cluster.u64 %0, [ra];\n\t}"
+                 : "=l"(v) : "r"(addr), "r"(rank), "r"(self));
     return v;
 }
 
-__global__ void __launch_bounds__(GOOD_BLOCK, 1)
+__global__ void __launch_bounds__(GOOD_BLOCK + 32, 1)
 good_cluster_kernel(const DevDesign *__restrict__ designs, const uint32_t *__restrict__ list,
                     uint32_t C_launch, uint32_t *err, uint32_t t_begin, uint32_t t_end) {
     extern __shared__ __align__(128) uint64_t gsm[];
@@ -352,81 +471,140 @@ good_cluster_kernel(const DevDesign *__restrict__ designs, const uint32_t *__res
     const uint32_t I = D.I, IR = I + D.R, n_net = D.n_net;
     const uint32_t T = min(D.T, t_end);
     if (t_begin >= T) return;   // the same in every CTA of the cluster
+    constexpr int KR = 5;       // registers a thread keeps the records of
     const uint32_t tid = threadIdx.x, B = blockDim.x;
-    const uint32_t own = D.cl_own, rown = D.cl_rown;
-    const size_t vwords = (size_t)own + 2 * (size_t)rown + I;
-    uint64_t *qv = gsm + own;            // [2][rown] register banks (node values [own] before)
-    uint64_t *inv = qv + 2 * rown;       // [I] inputs
-    const uint32_t c0 = D.cl_ch_off[rank], NC = D.cl_ch_off[rank + 1] - c0;
-    uint4 *ch = reinterpret_cast<uint4 *>(gsm + ((vwords + 1) & ~(size_t)1));   // [NC]
-    const uint4 *__restrict__ cdesc = D.cl_desc + (size_t)rank * own;
-    const uint4 *__restrict__ creg = D.cl_reg + D.cl_reg_off[rank];
-    const uint32_t NR = D.cl_reg_off[rank + 1] - D.cl_reg_off[rank];
+    const uint32_t own = D.cl_own, rown = D.cl_rown, S = D.cl_steps, W = D.cl_width;
+    uint64_t *const qv = gsm + own;            // [2][rown] register banks (node values [own] before)
+    uint64_t *const inv = qv + 2 * rown;       // [I] inputs
+    const uint32_t rfirst = D.cl_reg_off[rank], NR = D.cl_reg_off[rank + 1] - rfirst;
+    const uint4 *__restrict__ creg = D.cl_reg + rfirst;
+    const bool latch_sync = D.cl_latch_sync != 0u;
+    const uint64_t *__restrict__ stim = D.stim;
+    uint64_t *__restrict__ const rows = D.rows;
     const uint32_t base = smem_u32(gsm);
-    for (uint32_t c = tid; c < NC; c += B) ch[c] = D.cl_chunk[c0 + c];
+    for (uint32_t k = D.cl_const_off[rank] + tid; k < D.cl_const_off[rank + 1]; k += B) {
+        const uint4 g = D.cl_const[k];
+        gsm[g.x] = (uint64_t)g.z << 32 | g.y;
+    }
+    const uint64_t in_mask = tid < I ? wmask(D.net_w[tid]) : 0ull;
+    uint32_t gy[KR], gr[KR];   // D location; register | (64 - width) << 24
+#pragma unroll
+    for (int k = 0; k < KR; ++k) {
+        const uint4 g = tid + k * B < NR ? creg[tid + k * B] : make_uint4(0u, CL_SELF, 64u, 0u);
+        gy[k] = g.y;
+        gr[k] = g.x | (64u - g.z) << 24;
+    }
     // registers entering t_begin: the reset value, or the latch of the previous window
     for (uint32_t j = tid; j < NR; j += B) {
         const uint4 g = creg[j];
         uint64_t q = 0ull;
-        if (t_begin > 0) q = D.rows[(size_t)(t_begin - 1) * n_net + g.w] & wmask(g.z);
+        if (t_begin > 0) q = rows[(size_t)(t_begin - 1) * n_net + g.w] & wmask(g.z);
         qv[(t_begin & 1u) * rown + j] = q;
+        rows[(size_t)t_begin * n_net + I + g.x] = q;
     }
-    // all CTAs of the cluster are running and initialised before any remote read
-    cluster_sync();
-
-    uint32_t cf = 0;                             // chunk of the next prefetch (wraps)
-    auto prefetch = [&]() -> uint4 {
-        if (NC == 0) return make_uint4(0u, 0u, 0u, 0u);   // a design without nodes
-        const uint4 b = ch[cf];
-        cf = cf + 1 == NC ? 0 : cf + 1;
-        return tid < (b.y & 0x7FFFFFFFu) ? __ldg(cdesc + b.x + tid) : make_uint4(0u, 0u, 0u, 0u);
-    };
-    uint4 dq0 = prefetch();
-    uint4 dq1 = prefetch();
-    uint4 dq2 = prefetch();
-
-    for (uint32_t t = t_begin; t < T; ++t) {
-        uint64_t *row = D.rows + (size_t)t * n_net;
-        const uint32_t bank_off = (t & 1u) * rown;
-        // inputs of cycle t into this CTA's copy; CTA 0 writes them to the trace
-        for (uint32_t i = tid; i < I; i += B) {
-            const uint64_t v = __ldg(D.stim + (size_t)t * I + i) & wmask(D.net_w[i]);
+    // inputs of cycle t: every CTA's copy; CTA 0 writes them to the trace
+    uint64_t s_next = tid < I ? __ldg(stim + (size_t)t_begin * I + tid) : 0ull;
+    auto inputs = [&](uint32_t t) {
+        uint64_t *__restrict__ const row = rows + (size_t)t * n_net;
+        if (tid < I) {
+            const uint64_t v = s_next & in_mask;
+            if (t + 1 < T) s_next = __ldg(stim + (size_t)(t + 1) * I + tid);
+            inv[tid] = v;
+            if (rank == 0) row[tid] = v;
+        }
+        for (uint32_t i = tid + B; i < I; i += B) {
+            const uint64_t v = __ldg(stim + (size_t)t * I + i) & wmask(D.net_w[i]);
             inv[i] = v;
             if (rank == 0) row[i] = v;
         }
-        // this CTA's registers (a contiguous index range): Q of cycle t to the trace
-        for (uint32_t j = tid; j < NR; j += B) row[I + creg[j].x] = qv[bank_off + j];
-        __syncthreads();
+    };
+    inputs(t_begin);
+    // all CTAs of the cluster are running and initialised before any remote read
+    cluster_sync();
+
+    // Node records two steps ahead in registers (wrapping into the next cycle). The load has no
+    // condition: merging it with another value would wait for it at once. Threads without
+    // nodes read the blank record behind the last.
+    const uint32_t inc = tid < W ? W : 0u, END = S * W;
+    const uint4 *__restrict__ const cdesc = D.cl_desc + (tid < W ? (size_t)rank * END + tid : (size_t)C * END);
+    uint32_t off = 0;
+    auto prefetch = [&]() -> uint4 {
+        const uint4 d = __ldg(cdesc + off);
+        off = off + inc == END ? 0u : off + inc;
+        return d;
+    };
+    uint4 d0 = prefetch(), d1 = prefetch();
+
+    // Arrivals behind a CTA barrier: the last warp, which has no nodes, releases what the CTA's
+    // threads wrote before the barrier.
+    const bool releases = tid >= B - 32u;
+    auto arrive = [&]() { if (releases) cluster_arrive(); else cluster_arrive_relaxed(); };
+
+    for (uint32_t t = t_begin; t < T; ++t) {
+        uint64_t *__restrict__ const row = rows + (size_t)t * n_net + IR;
+        const uint32_t bank = (t & 1u) * rown * 8u;
         auto fetch = [&](uint32_t e) -> uint64_t {
-            const uint32_t w = (e & CL_WORD) + ((e & CL_REG) ? bank_off : 0u);
-            const uint32_t r = (e & CL_SELF) ? rank : ((e >> CL_RANK_SHIFT) & 15u);
-            return dsm_load(base + w * 8u, r);
+            const uint32_t a = base + (e & CL_WORD) * 8u + ((e & CL_REG) ? bank : 0u);
+            return dsm_load(a, (e >> CL_RANK_SHIFT) & 15u, e & CL_SELF);
         };
-        for (uint32_t c = 0; c < NC; ++c) {
-            const uint4 b = ch[c];
-            const uint4 d0 = dq0;
-            dq0 = dq1;
-            dq1 = dq2;
-            dq2 = prefetch();
-            if (tid < (b.y & 0x7FFFFFFFu)) {
-                const uint32_t op = meta_op(d0.w);
-                const int no = n_operands(op);
-                uint64_t a = 0, bb = 0, cc = 0;
-                if (no >= 1) a = fetch(d0.x);
-                if (no >= 2) bb = fetch(d0.y);
-                if (no >= 3) cc = fetch(d0.z);
-                const uint64_t v = eval_op(d0, a, bb, cc);
-                gsm[b.x + tid] = v;
-                row[IR + b.z + tid] = v;
+        auto step = [&](uint32_t s, uint4 &d) {
+            const uint4 e = d;
+            d = prefetch();
+            const bool on = (e.w & GM_VALID) != 0u;
+            uint64_t v = 0ull;
+            if (on) {
+                const uint64_t x = fetch(e.x), y = fetch(e.y);
+                uint64_t c = 0ull;
+                if (e.w & GM_MUX) c = fetch(e.z);
+                v = good_eval(e.w, x, y, c);
+                gsm[e.z >> CL_BITS | ((e.w >> CL_SLOT_HI) & 15u) << (32 - CL_BITS)] = v;
             }
-            if (b.y & 0x80000000u) cluster_sync();   // the level is complete cluster-wide
+            __syncthreads();
+            if (s > 0) cluster_wait();              // every CTA has done step s - 1
+            if (s + 1 < S || latch_sync) cluster_arrive_relaxed();
+            if (on) row[e.x >> CL_BITS | (e.y >> CL_BITS) << (32 - CL_BITS)] = v;
+        };
+        if (releases) {
+#pragma unroll 1
+            for (uint32_t s = 0; s < S; ++s) {
+                __syncthreads();
+                asm volatile("fence.acq_rel.cluster;" ::: "memory");
+                if (s > 0) cluster_wait();
+                if (s + 1 < S || latch_sync) cluster_arrive_relaxed();
+            }
+        } else {
+#pragma unroll 1
+            for (uint32_t s = 0; s < S; s += 2) {   // S is even
+                step(s, d0);
+                step(s + 1, d1);
+            }
         }
-        // latch: Q of cycle t+1 into the other bank
-        for (uint32_t j = tid; j < NR; j += B) {
+        if (latch_sync && S) cluster_wait();
+        // latch: Q of cycle t+1 into the other bank, and the next inputs once no latch reads these
+        const uint32_t nb = rown - (t & 1u) * rown;
+        uint64_t q[KR];
+#pragma unroll
+        for (int k = 0; k < KR; ++k)
+            if (tid + k * B < NR) q[k] = fetch(gy[k]) & (~0ull >> (gr[k] >> 24));
+#pragma unroll
+        for (int k = 0; k < KR; ++k)
+            if (tid + k * B < NR) qv[nb + tid + k * B] = q[k];
+        for (uint32_t j = tid + KR * B; j < NR; j += B) {
             const uint4 g = creg[j];
-            qv[(rown - bank_off) + j] = fetch(g.y) & wmask(g.z);
+            qv[nb + j] = fetch(g.y) & wmask(g.z);
         }
-        cluster_sync();
+        __syncthreads();
+        if (t + 1 < T) inputs(t + 1);
+        __syncthreads();
+        arrive();
+        if (t + 1 < T) {
+            uint64_t *__restrict__ const rq = rows + (size_t)(t + 1) * n_net + I;
+#pragma unroll
+            for (int k = 0; k < KR; ++k)
+                if (tid + k * B < NR) rq[gr[k] & 0xFFFFFFu] = q[k];
+            for (uint32_t j = tid + KR * B; j < NR; j += B) rq[creg[j].x] = qv[nb + j];
+        }
+        cluster_wait();
     }
 }
 
@@ -1892,6 +2070,7 @@ plain_kernel(const DevDesign *__restrict__ designs, uint32_t design, DevFaults f
 
 size_t good_smem_bytes(bool use_smem, uint32_t max_net, uint32_t max_reg, uint32_t max_chunks, bool staged) {
     const size_t vwords = use_smem ? (size_t)max_net + max_reg : 0;
+    if (use_smem && !staged) return vwords * sizeof(uint64_t);
     if (staged)
         return ((vwords + 1) & ~(size_t)1) * sizeof(uint64_t) + (size_t)GOOD_NSTAGE * GOOD_BLOCK * 16 +
                (size_t)max_chunks * sizeof(uint2);
@@ -1915,25 +2094,19 @@ cudaError_t launch_good_trace(const DevDesign *d_designs, const uint32_t *design
         return cudaLaunchKernel(fn, dim3(n_list), dim3(GOOD_BLOCK + 32), args, smem, stream);
     }
     if (use_smem) {
-        e = cudaFuncSetAttribute(good_trace_kernel<true>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = cudaFuncSetAttribute(good_trace_smem_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        good_trace_kernel<true><<<n_list, GOOD_BLOCK, smem, stream>>>(d_designs, design_list, max_net,
-                                                                     max_reg, max_chunks,
-                                                                     t_begin, t_end);
+        good_trace_smem_kernel<4><<<n_list, GOOD_BLOCK, smem, stream>>>(d_designs, design_list, max_net, t_begin, t_end);
     } else {
-        e = cudaFuncSetAttribute(good_trace_kernel<false>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = cudaFuncSetAttribute(good_trace_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        good_trace_kernel<false><<<n_list, GOOD_BLOCK, smem, stream>>>(d_designs, design_list, 0, 0,
-                                                                      max_chunks, t_begin, t_end);
+        good_trace_kernel<<<n_list, GOOD_BLOCK, smem, stream>>>(d_designs, design_list, t_begin, t_end);
     }
     return cudaGetLastError();
 }
 
-size_t good_cluster_smem_bytes(uint32_t own, uint32_t rown, uint32_t n_inputs, uint32_t max_chunks) {
-    const size_t vwords = (size_t)own + 2 * (size_t)rown + n_inputs;
-    return ((vwords + 1) & ~(size_t)1) * sizeof(uint64_t) + (size_t)max_chunks * 16;
+size_t good_cluster_smem_bytes(uint32_t own, uint32_t rown, uint32_t n_inputs) {
+    return ((size_t)own + 2 * (size_t)rown + n_inputs) * sizeof(uint64_t);
 }
 
 static cudaError_t good_cluster_attrs(uint32_t C, size_t smem) {
@@ -1943,7 +2116,7 @@ static cudaError_t good_cluster_attrs(uint32_t C, size_t smem) {
     return e;
 }
 
-int good_cluster_max_active(uint32_t C, size_t smem) {
+int good_cluster_max_active(uint32_t C, uint32_t threads, size_t smem) {
     if (good_cluster_attrs(C, smem) != cudaSuccess) { cudaGetLastError(); return 0; }
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
@@ -1952,7 +2125,7 @@ int good_cluster_max_active(uint32_t C, size_t smem) {
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
     cfg.gridDim = dim3(C);
-    cfg.blockDim = dim3(GOOD_BLOCK);
+    cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.attrs = at;
     cfg.numAttrs = 1;
@@ -1965,7 +2138,7 @@ int good_cluster_max_active(uint32_t C, size_t smem) {
 }
 
 cudaError_t launch_good_cluster(const DevDesign *d_designs, const uint32_t *design_list,
-                                uint32_t n_list, uint32_t C, size_t smem, uint32_t *err,
+                                uint32_t n_list, uint32_t C, uint32_t threads, size_t smem, uint32_t *err,
                                 cudaStream_t stream, uint32_t t_begin, uint32_t t_end) {
     if (n_list == 0) return cudaSuccess;
     cudaError_t e = good_cluster_attrs(C, smem);
@@ -1977,7 +2150,7 @@ cudaError_t launch_good_cluster(const DevDesign *d_designs, const uint32_t *desi
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
     cfg.gridDim = dim3(n_list * C);
-    cfg.blockDim = dim3(GOOD_BLOCK);
+    cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cfg.attrs = at;
