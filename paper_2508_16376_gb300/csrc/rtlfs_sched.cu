@@ -68,7 +68,7 @@ __device__ __forceinline__ void load_params(const __nv_bfloat16 *__restrict__ wb
 // One thread per sample; weights (as FP32 copies of the BF16 values) in shared memory.
 __global__ void mlp_forward_kernel(const __nv_bfloat16 *__restrict__ wb, const float *__restrict__ X,
                                    uint32_t n, float *y) {
-    __shared__ float sw[MLP_PARAMS];
+    __shared__ __align__(16) float sw[MLP_PARAMS];
     load_params(wb, sw);
     __syncthreads();
     const uint32_t s = blockIdx.x * blockDim.x + threadIdx.x;
@@ -87,108 +87,239 @@ __global__ void mlp_forward_kernel(const __nv_bfloat16 *__restrict__ wb, const f
         h1[j] = a > 0.f ? a : 0.f;
     }
     float out = sw[MLP_OFF_B3];
-    for (int j = 0; j < MLP_H; ++j) {
-        float a = b2[j];
+#pragma unroll 1
+    for (int j = 0; j < MLP_H; j += 4) {   // four units per 16-byte read of W2, the same for all lanes
+        float a[4] = {b2[j], b2[j + 1], b2[j + 2], b2[j + 3]};
 #pragma unroll
-        for (int i = 0; i < MLP_H; ++i) a = fmaf(h1[i], W2[i * MLP_H + j], a);
-        a = a > 0.f ? a : 0.f;
-        out = fmaf(a, w3[j], out);
+        for (int i = 0; i < MLP_H; ++i) {
+            const float4 w = *reinterpret_cast<const float4 *>(W2 + i * MLP_H + j);
+            a[0] = fmaf(h1[i], w.x, a[0]);
+            a[1] = fmaf(h1[i], w.y, a[1]);
+            a[2] = fmaf(h1[i], w.z, a[2]);
+            a[3] = fmaf(h1[i], w.w, a[3]);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) out = fmaf(a[k] > 0.f ? a[k] : 0.f, w3[j + k], out);
     }
     y[s] = out;
 }
 
-// Forward + backward of the mean squared error over n samples for one tile of MLP_TILE
-// samples per CTA; the tile's parameter gradients are added into grad (FP32 atomics) and
-// its squared errors into loss_sum.
-__global__ void __launch_bounds__(256)
+// Forward + backward of the mean squared error over n samples. A CTA walks tiles of 16 * SPT samples;
+// its three 64-wide products per tile (layer 2, its input gradient, the gradient of W2) are register
+// tiled: thread (ty, tx) holds SPT consecutive samples x the four units tx + 16 k, or the 4 x 4 block
+// of W2's gradient, whose rows it keeps in registers over all tiles, as the other gradients, and
+// adds to grad once (FP32 atomics; squared errors into loss_sum). Activations lie by unit and then
+// sample, padded by four: both kinds of read are 16-byte loads without bank conflicts.
+// Bound by the FP32 multiply-adds (1.8 GFLOP of them at 65537 samples). One output per thread with
+// two shared loads per multiply-add, and an atomic per parameter and tile of 64 samples and per
+// sample's error, made a call with 65537 samples 440 us; it is 123 so, half of it the copies.
+template <int SPT> struct GradVec { float v[SPT]; };
+template <int SPT> __device__ __forceinline__ GradVec<SPT> ld_vec(const float *p) {
+    GradVec<SPT> r;
+    if constexpr (SPT == 2) {
+        const float2 a = *reinterpret_cast<const float2 *>(p);
+        r.v[0] = a.x; r.v[1] = a.y;
+    } else {
+#pragma unroll
+        for (int k = 0; k < SPT; k += 4) {
+            const float4 a = *reinterpret_cast<const float4 *>(p + k);
+            r.v[k] = a.x; r.v[k + 1] = a.y; r.v[k + 2] = a.z; r.v[k + 3] = a.w;
+        }
+    }
+    return r;
+}
+template <int SPT> __device__ __forceinline__ void st_vec(float *p, const GradVec<SPT> &r) {
+    if constexpr (SPT == 2) {
+        *reinterpret_cast<float2 *>(p) = make_float2(r.v[0], r.v[1]);
+    } else {
+#pragma unroll
+        for (int k = 0; k < SPT; k += 4) *reinterpret_cast<float4 *>(p + k) = make_float4(r.v[k], r.v[k + 1], r.v[k + 2], r.v[k + 3]);
+    }
+}
+
+constexpr int GRAD_W1 = 2 * MLP_H * MLP_H;   // shared floats: W2 by rows and by columns, then
+constexpr int GRAD_B1 = GRAD_W1 + MLP_IN * MLP_H, GRAD_B2 = GRAD_B1 + MLP_H, GRAD_W3 = GRAD_B2 + MLP_H;
+constexpr int GRAD_B3 = GRAD_W3 + MLP_H, GRAD_ACT = GRAD_B3 + 4;
+template <int SPT> constexpr int grad_floats() { return GRAD_ACT + 2 * MLP_H * (16 * SPT + 4) + MLP_IN * 16 * SPT; }
+
+template <int SPT>
+__global__ void __launch_bounds__(256, 2)
 mlp_grad_kernel(const __nv_bfloat16 *__restrict__ wb, const float *__restrict__ X,
                 const float *__restrict__ tgt, uint32_t n, float *grad, float *loss_sum) {
-    extern __shared__ float gsh[];
-    float *sw = gsh;                                   // [MLP_PARAMS]
-    float *h1 = sw + MLP_PARAMS;                       // [TILE][H]  post-activation
-    float *h2 = h1 + MLP_TILE * MLP_H;                 // [TILE][H]  post-activation
-    float *d2 = h2 + MLP_TILE * MLP_H;                 // [TILE][H]  dL/d(pre-activation 2)
-    float *d1 = d2 + MLP_TILE * MLP_H;                 // [TILE][H]  dL/d(pre-activation 1)
-    float *xs = d1 + MLP_TILE * MLP_H;                 // [TILE][IN]
-    float *dy = xs + MLP_TILE * MLP_IN;                // [TILE]
-    load_params(wb, sw);
-    const float *W1 = sw, *b1 = sw + MLP_OFF_B1, *W2 = sw + MLP_OFF_W2, *b2 = sw + MLP_OFF_B2;
-    const float *w3 = sw + MLP_OFF_W3;
-    const uint32_t s0 = blockIdx.x * MLP_TILE, tid = threadIdx.x, B = blockDim.x;
-    for (uint32_t k = tid; k < MLP_TILE * MLP_IN; k += B) {
-        const uint32_t s = s0 + k / MLP_IN;
-        xs[k] = s < n ? X[(size_t)s0 * MLP_IN + k] : 0.f;
-    }
-    __syncthreads();
-    // layer 1
-    for (uint32_t k = tid; k < MLP_TILE * MLP_H; k += B) {
-        const uint32_t s = k / MLP_H, j = k % MLP_H;
-        float a = b1[j];
-        for (int i = 0; i < MLP_IN; ++i) a = fmaf(xs[s * MLP_IN + i], W1[i * MLP_H + j], a);
-        h1[k] = a > 0.f ? a : 0.f;
-    }
-    __syncthreads();
-    // layer 2
-    for (uint32_t k = tid; k < MLP_TILE * MLP_H; k += B) {
-        const uint32_t s = k / MLP_H, j = k % MLP_H;
-        float a = b2[j];
-        for (int i = 0; i < MLP_H; ++i) a = fmaf(h1[s * MLP_H + i], W2[i * MLP_H + j], a);
-        h2[k] = a > 0.f ? a : 0.f;
-    }
-    __syncthreads();
-    // output, error and dL/dy = 2 (y - t) / n
-    if (tid < MLP_TILE) {
-        const uint32_t s = s0 + tid;
-        float e = 0.f;
-        if (s < n) {
-            float out = sw[MLP_OFF_B3];
-            for (int j = 0; j < MLP_H; ++j) out = fmaf(h2[tid * MLP_H + j], w3[j], out);
-            e = out - tgt[s];
-            atomicAdd(loss_sum, e * e);
+    constexpr int H = MLP_H, S = 16 * SPT, LD = S + 4;
+    static_assert(H == 64, "16 x 16 threads hold four units each");
+    extern __shared__ __align__(16) float gsh[];
+    float *const w2r = gsh, *const w2c = gsh + H * H;   // [i][4 tx + k] = W2[i][tx + 16 k]; [j][4 tx + k] = W2[tx + 16 k][j]
+    float *const W1 = gsh + GRAD_W1, *const b1 = gsh + GRAD_B1, *const b2 = gsh + GRAD_B2, *const w3 = gsh + GRAD_W3;
+    float *const h1 = gsh + GRAD_ACT, *const d2 = h1 + H * LD, *const xs = d2 + H * LD;   // [unit][LD], [input][S]
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    for (int k = tid; k < MLP_PARAMS; k += 256) {
+        const float w = __bfloat162float(wb[k]);
+        if (k >= MLP_OFF_W2 && k < MLP_OFF_B2) {
+            const int i = (k - MLP_OFF_W2) / H, j = (k - MLP_OFF_W2) % H;
+            w2r[i * H + (j & 15) * 4 + (j >> 4)] = w;
+            w2c[j * H + (i & 15) * 4 + (i >> 4)] = w;
+        } else if (k < MLP_OFF_W2) {
+            W1[k] = w;   // W1, b1
+        } else {
+            b2[k - MLP_OFF_B2] = w;   // b2, w3, b3
         }
-        dy[tid] = 2.f * e / (float)n;
     }
-    __syncthreads();
-    for (uint32_t k = tid; k < MLP_TILE * MLP_H; k += B) {
-        const uint32_t s = k / MLP_H, j = k % MLP_H;
-        d2[k] = h2[k] > 0.f ? w3[j] * dy[s] : 0.f;
-    }
-    __syncthreads();
-    for (uint32_t k = tid; k < MLP_TILE * MLP_H; k += B) {
-        const uint32_t s = k / MLP_H, i = k % MLP_H;
-        float a = 0.f;
-        for (int j = 0; j < MLP_H; ++j) a = fmaf(W2[i * MLP_H + j], d2[s * MLP_H + j], a);
-        d1[k] = h1[k] > 0.f ? a : 0.f;
-    }
-    __syncthreads();
-    // parameter gradients of this tile
-    for (uint32_t k = tid; k < MLP_H * MLP_H; k += B) {          // W2
-        const uint32_t i = k / MLP_H, j = k % MLP_H;
-        float a = 0.f;
-        for (uint32_t s = 0; s < MLP_TILE; ++s) a = fmaf(h1[s * MLP_H + i], d2[s * MLP_H + j], a);
-        atomicAdd(grad + MLP_OFF_W2 + k, a);
-    }
-    for (uint32_t k = tid; k < MLP_IN * MLP_H; k += B) {         // W1
-        const uint32_t i = k / MLP_H, j = k % MLP_H;
-        float a = 0.f;
-        for (uint32_t s = 0; s < MLP_TILE; ++s) a = fmaf(xs[s * MLP_IN + i], d1[s * MLP_H + j], a);
-        atomicAdd(grad + k, a);
-    }
-    for (uint32_t j = tid; j < MLP_H; j += B) {                  // b1, b2, w3
-        float g1 = 0.f, g2 = 0.f, g3 = 0.f;
-        for (uint32_t s = 0; s < MLP_TILE; ++s) {
-            g1 += d1[s * MLP_H + j];
-            g2 += d2[s * MLP_H + j];
-            g3 = fmaf(h2[s * MLP_H + j], dy[s], g3);
+    float g2[4][4] = {}, g1[MLP_IN][4] = {}, gb1[4] = {}, gb2[4] = {}, gw3[4] = {}, gb3 = 0.f, loss = 0.f;
+    const uint32_t tiles = n / S + (n % S != 0);
+    for (uint32_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const uint32_t s0 = tile * S;
+        __syncthreads();   // the last tile's reads, and the weights
+        for (int k = tid; k < S * MLP_IN; k += 256) {
+            const int s = k / MLP_IN;
+            xs[(k % MLP_IN) * S + s] = s0 + s < n ? X[(size_t)s0 * MLP_IN + k] : 0.f;
         }
-        atomicAdd(grad + MLP_OFF_B1 + j, g1);
-        atomicAdd(grad + MLP_OFF_B2 + j, g2);
-        atomicAdd(grad + MLP_OFF_W3 + j, g3);
+        __syncthreads();
+        for (int k = tid; k < S * H; k += 256) {   // layer 1
+            const int j = k / S, s = k % S;
+            float a = b1[j];
+#pragma unroll
+            for (int i = 0; i < MLP_IN; ++i) a = fmaf(xs[i * S + s], W1[i * H + j], a);
+            h1[j * LD + s] = a > 0.f ? a : 0.f;
+        }
+        float t[SPT];
+#pragma unroll
+        for (int p = 0; p < SPT; ++p) t[p] = s0 + ty * SPT + p < n ? tgt[s0 + ty * SPT + p] : 0.f;
+        __syncthreads();
+        float acc[SPT][4];
+#pragma unroll
+        for (int p = 0; p < SPT; ++p)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) acc[p][k] = b2[tx + 16 * k];
+#pragma unroll 4
+        for (int i = 0; i < H; ++i) {   // layer 2
+            const GradVec<SPT> a = ld_vec<SPT>(h1 + i * LD + ty * SPT);
+            const GradVec<4> w = ld_vec<4>(w2r + i * H + tx * 4);
+#pragma unroll
+            for (int p = 0; p < SPT; ++p)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) acc[p][k] = fmaf(a.v[p], w.v[k], acc[p][k]);
+        }
+        // output, error and dL/dy = 2 (y - t) / n; dL/d(pre-activation 2)
+        float dy[SPT];
+#pragma unroll
+        for (int p = 0; p < SPT; ++p) {
+            float out = 0.f;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                acc[p][k] = acc[p][k] > 0.f ? acc[p][k] : 0.f;
+                out = fmaf(acc[p][k], w3[tx + 16 * k], out);
+            }
+#pragma unroll
+            for (int o = 8; o; o >>= 1) out += __shfl_xor_sync(0xFFFFFFFFu, out, o);
+            const float e = s0 + ty * SPT + p < n ? out + gsh[GRAD_B3] - t[p] : 0.f;
+            dy[p] = 2.f * e / (float)n;
+            if (tx == 0) {
+                loss = fmaf(e, e, loss);
+                gb3 += dy[p];
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            GradVec<SPT> d;
+#pragma unroll
+            for (int p = 0; p < SPT; ++p) {
+                d.v[p] = acc[p][k] > 0.f ? w3[tx + 16 * k] * dy[p] : 0.f;
+                gb2[k] += d.v[p];
+                gw3[k] = fmaf(acc[p][k], dy[p], gw3[k]);
+            }
+            st_vec<SPT>(d2 + (tx + 16 * k) * LD + ty * SPT, d);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int p = 0; p < SPT; ++p)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) acc[p][k] = 0.f;
+#pragma unroll 4
+        for (int j = 0; j < H; ++j) {   // dL/d(activation 1)
+            const GradVec<SPT> a = ld_vec<SPT>(d2 + j * LD + ty * SPT);
+            const GradVec<4> w = ld_vec<4>(w2c + j * H + tx * 4);
+#pragma unroll
+            for (int p = 0; p < SPT; ++p)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) acc[p][k] = fmaf(w.v[k], a.v[p], acc[p][k]);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const GradVec<SPT> a = ld_vec<SPT>(h1 + (tx + 16 * k) * LD + ty * SPT);
+#pragma unroll
+            for (int p = 0; p < SPT; ++p) {
+                acc[p][k] = a.v[p] > 0.f ? acc[p][k] : 0.f;
+                gb1[k] += acc[p][k];
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < MLP_IN; ++i) {
+            const GradVec<SPT> x = ld_vec<SPT>(xs + i * S + ty * SPT);
+#pragma unroll
+            for (int p = 0; p < SPT; ++p)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) g1[i][k] = fmaf(x.v[p], acc[p][k], g1[i][k]);
+        }
+#pragma unroll 2
+        for (int s = 0; s < S; s += 4) {   // W2, rows ty + 16 i
+            GradVec<4> a[4], d[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                a[k] = ld_vec<4>(h1 + (ty + 16 * k) * LD + s);
+                d[k] = ld_vec<4>(d2 + (tx + 16 * k) * LD + s);
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) g2[i][k] = fmaf(a[i].v[q], d[k].v[q], g2[i][k]);
+        }
     }
-    if (tid == 0) {
-        float g = 0.f;
-        for (uint32_t s = 0; s < MLP_TILE; ++s) g += dy[s];
-        atomicAdd(grad + MLP_OFF_B3, g);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) atomicAdd(grad + MLP_OFF_W2 + (ty + 16 * i) * H + tx + 16 * k, g2[i][k]);
+    // the rest over the 16 rows of threads: a warp's two, then the eight warps
+    constexpr int V = 4 * (MLP_IN + 3);
+    float *const red = h1;   // [8][16][V]
+    static_assert(8 * 16 * V <= 2 * H * LD, "the reduction lies over the activations");
+    __syncthreads();
+    float own[V];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+#pragma unroll
+        for (int i = 0; i < MLP_IN; ++i) own[4 * i + k] = g1[i][k];
+        own[4 * MLP_IN + k] = gb1[k];
+        own[4 * MLP_IN + 4 + k] = gb2[k];
+        own[4 * MLP_IN + 8 + k] = gw3[k];
+    }
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+        own[v] += __shfl_xor_sync(0xFFFFFFFFu, own[v], 16);
+        if (tid % 32 < 16) red[((tid >> 5) * V + v) * 16 + tx] = own[v];
+    }
+    loss += __shfl_xor_sync(0xFFFFFFFFu, loss, 16);
+    gb3 += __shfl_xor_sync(0xFFFFFFFFu, gb3, 16);
+    if (tid % 32 == 0) {
+        gsh[2 * (tid >> 5)] = loss;   // over the weights, whose last reads lie before the barrier
+        gsh[2 * (tid >> 5) + 1] = gb3;
+    }
+    __syncthreads();
+    for (int k = tid; k < 16 * V; k += 256) {
+        const int v = k >> 4, u = (k & 15) + 16 * (v & 3), what = v >> 2;   // unit; input, b1, b2, w3
+        float a = 0.f;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) a += red[w * V * 16 + k];
+        const int at = what < MLP_IN ? what * H : what == MLP_IN ? MLP_OFF_B1 : what == MLP_IN + 1 ? MLP_OFF_B2 : MLP_OFF_W3;
+        atomicAdd(grad + at + u, a);
+    }
+    if (tid < 2) {
+        float a = 0.f;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) a += gsh[2 * w + tid];
+        atomicAdd(tid == 0 ? loss_sum : grad + MLP_OFF_B3, a);
     }
 }
 
@@ -330,18 +461,18 @@ cudaError_t launch_mlp_forward(const void *wb, const float *X, uint32_t n, float
     return cudaGetLastError();
 }
 
-size_t mlp_grad_smem() {
-    return (MLP_PARAMS + 4 * MLP_TILE * MLP_H + MLP_TILE * MLP_IN + MLP_TILE) * sizeof(float);
-}
-
 cudaError_t launch_mlp_grad(const void *wb, const float *X, const float *t, uint32_t n, float *grad,
                             float *loss_sum, cudaStream_t s) {
     if (!n) return cudaSuccess;
-    const size_t smem = mlp_grad_smem();
-    cudaError_t e = cudaFuncSetAttribute(mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // Tiles of 128 samples when they fill the 152 SMs, else of 32, for more CTAs; two CTAs per SM
+    // (65537 samples, the call: 123 us; one CTA per SM 127-135, tiles of 64 126).
+    const bool big = n >= 152u * 128u;
+    const uint32_t S = big ? 128 : 32, tiles = n / S + (n % S != 0), grid = tiles < 304u ? tiles : 304u;
+    const size_t smem = (big ? grad_floats<8>() : grad_floats<2>()) * sizeof(float);
+    const auto fn = big ? mlp_grad_kernel<8> : mlp_grad_kernel<2>;
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    mlp_grad_kernel<<<(n + MLP_TILE - 1) / MLP_TILE, 256, smem, s>>>((const __nv_bfloat16 *)wb, X, t, n,
-                                                                     grad, loss_sum);
+    fn<<<grid, 256, smem, s>>>((const __nv_bfloat16 *)wb, X, t, n, grad, loss_sum);
     return cudaGetLastError();
 }
 

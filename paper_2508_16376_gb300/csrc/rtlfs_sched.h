@@ -6,7 +6,6 @@ namespace rtlfs {
 
 constexpr int MLP_IN = 5;       // cone size, level, register depth to outputs, width, toggle rate
 constexpr int MLP_H = 64;
-constexpr int MLP_TILE = 64;    // samples per CTA in the gradient kernel
 constexpr int MLP_OFF_B1 = MLP_IN * MLP_H;              // 320
 constexpr int MLP_OFF_W2 = MLP_OFF_B1 + MLP_H;          // 384
 constexpr int MLP_OFF_B2 = MLP_OFF_W2 + MLP_H * MLP_H;  // 4480
@@ -21,7 +20,6 @@ constexpr uint32_t TOGGLE_CYCLES = 256;
 cudaError_t launch_features(const DevDesign *d_designs, DevFaults f, const float *const *net_static,
                             float *X, float *heur, cudaStream_t s, uint32_t t_limit = TOGGLE_CYCLES);
 cudaError_t launch_mlp_forward(const void *wb, const float *X, uint32_t n, float *y, cudaStream_t s);
-size_t mlp_grad_smem();
 cudaError_t launch_mlp_grad(const void *wb, const float *X, const float *t, uint32_t n, float *grad,
                             float *loss_sum, cudaStream_t s);
 cudaError_t launch_mlp_adam(float *master, void *wb, float *grad, float *m, float *v, float lr,
