@@ -387,14 +387,15 @@ int rtlfs_mlp_train(rtlfs_ctx *ctx, const float *X, const float *t, uint32_t n, 
  *
  * Scratch: a file-scope device array of RTLFS_STATIC_SCRATCH_BYTES (64 MiB) inside the
  * library, held by every GPU that loads the library until the process exits. A design
- * needs 4 B per net once plus 12 B per net + 8 B per node + 24 B per register for every
- * simultaneously simulated fault (faults run in waves that fit); a design whose single
+ * needs 4 B per net once plus at most 12 B per net + 8 B per node + 24 B per register for every
+ * simultaneously simulated fault (as many run at a time as fit); a design whose single
  * fault does not fit is rejected with RTLFS_E_ARG. Every call shares the array and leaves
  * its contents behind; the call clears what must start at zero. Calls whose work overlaps
  * on the GPU (other threads, other streams) race on the array: serialise them.
  *
  * What a call does: it copies the design's net-number map (4 B per net) from host memory
- * into the array, clears the wave's scratch, launches the kernel once per wave on `stream`
+ * into the array, launches the kernel on `stream` (once; for a design of more than some 1.8
+ * million nets and nodes once per wave of faults, after clearing the wave's scratch)
  * (a cudaStream_t; null = the legacy default stream), copies a 4-byte error word back to
  * the host and waits for `stream` before it returns. The first call on a device also looks
  * up the array's device address (cudaGetSymbolAddress) and keeps it; make that first call

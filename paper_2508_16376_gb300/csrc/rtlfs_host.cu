@@ -2465,7 +2465,17 @@ int rtlfs_fault_sim_static(rtlfs_ctx *ctx, uint32_t design_id, const rtlfs_fault
     CU(cudaMemcpyAsync(arena + L.ext2int_off, D.ext2int.data(), (size_t)4 * D.n_net,
                        cudaMemcpyHostToDevice, s));
     CU(cudaMemsetAsync(arena + L.err_off, 0, 8, s));
-    for (uint32_t first = 0; first < n_faults; first += wave) {
+    // a warp per fault where a design's bitmaps fit in its shared memory (up to some 1.8 million
+    // nets and nodes together), with less scratch than the other form's thread
+    const int warps = static_warps(D.N, D.n_net);
+    if (warps > 0) {
+        L.per_thread = ((size_t)8 * L.sn + (size_t)24 * L.sreg + 15) & ~(size_t)15;
+        const size_t slots = std::min<size_t>((STATIC_SCRATCH_BYTES - L.thread_off) / L.per_thread, n_faults);
+        const uint32_t per = (uint32_t)std::min<size_t>(warps, slots);
+        const uint32_t blocks = (uint32_t)std::min<size_t>(slots / per, (size_t)16 * ctx->n_sm);
+        CU(launch_static(ctx->d_designs.p, design_id, D.N, D.n_net, faults, results, n_faults, blocks, per, arena, L, s));
+    }
+    for (uint32_t first = 0; warps == 0 && first < n_faults; first += wave) {
         const uint32_t cnt = std::min(wave, n_faults - first);
         // value stamps and queued stamps must start at zero for every thread of the wave
         CU(cudaMemsetAsync(arena + L.thread_off, 0, (size_t)cnt * L.per_thread, s));

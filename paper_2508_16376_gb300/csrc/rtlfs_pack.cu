@@ -81,31 +81,6 @@ __device__ __forceinline__ PackSmem pack_layout(unsigned char *sm) {
     return m;
 }
 
-// eval_op with the operands in their value slots (x, y; s: the MUX2 select), without branches:
-// the lanes of a warp hold nodes of any op. x is shifted first (by 0 for most ops); the logic
-// ops, the shifts, CONCAT and MUX2 are then (x & y & A) ^ (x & B) ^ (y & C) ^ D with masks the
-// record names (PM_*), a MUX2's B and C chosen by s.
-__device__ __forceinline__ uint64_t pack_eval(uint4 d, uint64_t x, uint64_t y, uint64_t s) {
-    uint32_t w = d.w;
-    if (s) w ^= PM_B | PM_C;
-    const uint32_t k = meta_k(w), op = meta_op(w);
-    uint64_t xl, xr;   // shl/shr by more than 63 give 0
-    asm("shl.b64 %0, %1, %2;" : "=l"(xl) : "l"(x), "r"(k));
-    asm("shr.u64 %0, %1, %2;" : "=l"(xr) : "l"(x), "r"(k));
-    const uint64_t xs = w & PM_LEFT ? xl : xr;
-    auto mask = [&](uint32_t bit) -> uint64_t {
-        const uint32_t m = w & bit ? ~0u : 0u;
-        return (uint64_t)m << 32 | m;
-    };
-    uint64_t r = (xs & y & mask(PM_A)) ^ (xs & mask(PM_B)) ^ (y & mask(PM_C)) ^ mask(PM_D);
-    const uint64_t neg = op == OP_SUB ? ~0ull : 0ull;
-    r = w & PM_SUM ? x + (y ^ neg) - neg : r;
-    const bool cmp = op == OP_EQ ? x == y : x < y;
-    r = w & PM_CMP ? (cmp ? 1ull : 0ull) : r;
-    r = op == OP_CONST ? (uint64_t)d.y << 32 | d.x : r;
-    return r & (~0ull >> (64u - meta_w(w)));
-}
-
 // Compare-and-swap of an empty key where `on`; PK_EMPTY when it was empty or not on. Without
 // a branch around it.
 __device__ __forceinline__ uint32_t cas_if(bool on, uint32_t *key, uint32_t w) {

@@ -1,6 +1,6 @@
-// rtlfs_static.cu -- allocation-free fault simulation: a variant of the plain
-// one-thread-per-fault kernel whose per-thread scratch lives in one file-scope device
-// array instead of memory obtained from cudaMalloc.
+// rtlfs_static.cu -- allocation-free fault simulation: kernels with a warp, or for very large
+// designs a thread, per fault, whose scratch lives in one file-scope device array instead of
+// memory obtained from cudaMalloc.
 //
 // Who needs it: callers that cannot obtain device memory from cudaMalloc where they run --
 // a process whose device memory is owned by another allocator (a framework's caching pool
@@ -12,9 +12,10 @@
 // The array below is part of the library image: every GPU that loads the library keeps
 // its 64 MiB until the process exits. Every call shares it, it keeps the contents the last
 // call left, and two calls whose work overlaps on the GPU race on it.
-#include "rtlfs_internal.h"
+#include "rtlfs_device.h"
 #include "rtlfs_static.h"
 
+#include <algorithm>
 #include <mutex>
 
 namespace rtlfs {
@@ -44,38 +45,240 @@ cudaError_t static_scratch_address(int device, void **out) {
     return cudaSuccess;
 }
 
-__device__ __forceinline__ uint64_t s_wmask(uint32_t w) {
-    return w >= 64 ? ~0ull : ((1ull << w) - 1ull);
-}
-
-__device__ __forceinline__ int s_nops(uint32_t op) {
-    return op == OP_CONST ? 0
-         : (op == OP_NOT || op == OP_SHL || op == OP_SHR || op == OP_SLICE) ? 1
-         : op == OP_MUX2 ? 3 : 2;
-}
-
-__device__ __forceinline__ uint64_t s_eval(uint4 d, uint64_t a, uint64_t b, uint64_t c) {
-    const uint32_t m = d.w, k = meta_k(m);
-    uint64_t r;
-    switch (meta_op(m)) {
-    case OP_AND:    r = a & b; break;
-    case OP_OR:     r = a | b; break;
-    case OP_XOR:    r = a ^ b; break;
-    case OP_NOT:    r = ~a; break;
-    case OP_ADD:    r = a + b; break;
-    case OP_SUB:    r = a - b; break;
-    case OP_MUX2:   r = a ? b : c; break;
-    case OP_EQ:     r = (a == b) ? 1ull : 0ull; break;
-    case OP_LT:     r = (a < b) ? 1ull : 0ull; break;
-    case OP_SHL:    r = k >= 64 ? 0ull : (a << k); break;
-    case OP_SHR:
-    case OP_SLICE:  r = k >= 64 ? 0ull : (a >> k); break;
-    case OP_CONCAT: r = (k >= 64 ? 0ull : (a << k)) | b; break;
-    default:        r = ((uint64_t)d.y << 32) | d.x; break;
+// A fault that no context ever checked: false, with the result that says so, if it is out of range.
+__device__ __forceinline__ bool static_site(const DevDesign &D, const uint32_t *ext2int, const StaticFault &fx, uint32_t *err,
+                                            StaticResult *out, uint32_t *site) {
+    out->cycle = -1;
+    out->port = -1;
+    out->detected = 0;
+    out->reserved[0] = out->reserved[1] = out->reserved[2] = 0;
+    if (fx.net < D.n_net && fx.stuck <= 1) {
+        *site = ext2int[fx.net];
+        if (fx.bit < D.net_w[*site]) return true;
     }
-    return r & s_wmask(meta_w(m));
+    atomicOr(err, 1u);
+    out->detected = 254;
+    return false;
 }
 
+// Shared memory of one warp of static_kernel.
+struct StaticWarp {
+    uint32_t *bm, *top;      // dirty nodes, and the words of bm that hold one
+    uint32_t *df, *dtop;     // nets that differ this cycle, and the words of df that hold one
+    uint32_t *n_new;         // registers latched with a difference
+    uint16_t *list;          // [1024] a level's dirty nodes in 32 words of bm
+};
+
+__host__ __device__ inline uint32_t static_words(uint32_t n) { return (n + 31) / 32; }
+__host__ __device__ inline size_t static_warp_bytes(uint32_t n_node, uint32_t n_net) {
+    const uint32_t a = static_words(n_node), b = static_words(n_net);
+    return 4 * ((size_t)a + static_words(a) + b + static_words(b) + 4) + 2048;
+}
+
+// One warp per fault; a warp takes the next fault when it is done with one. A cycle in which the
+// machine has no register difference and the site's good bit is the stuck value is skipped
+// (32 cycles a look); in the others the warp takes the lowest level that has dirty nodes, its
+// lanes a node each, until none is left. Which nets differ is a bitmap in shared memory, so an
+// operand is one load, of the faulty value (in the slot's part of the scratch array) or of the
+// good one. What bounds it is the chain of a level, some 1000 cycles: the search for its nodes,
+// their 128-byte records, their operands. 1500 faults of 1200 nodes over 300 cycles: 13.0 ms with a
+// thread per fault and its heap of dirty nodes in the scratch array, 4.0 so.
+__global__ void __launch_bounds__(128)
+static_kernel(const DevDesign *__restrict__ designs, uint32_t design, const StaticFault *__restrict__ faults,
+              StaticResult *results, uint32_t n_faults, unsigned char *arena, StaticLayout L) {
+    extern __shared__ __align__(16) unsigned char ssm[];
+    constexpr uint32_t FULL = 0xFFFFFFFFu;
+    const DevDesign &D = designs[design];
+    const uint32_t I = D.I, IR = D.I + D.R, T = D.T, n_net = D.n_net, lane = threadIdx.x & 31u;
+    const uint32_t nw = static_words(D.N), nt = static_words(nw), dw = static_words(n_net), dt = static_words(dw);
+    const uint32_t slot = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    StaticWarp m;
+    m.bm = reinterpret_cast<uint32_t *>(ssm + (threadIdx.x >> 5) * static_warp_bytes(D.N, n_net));
+    m.top = m.bm + nw;
+    m.df = m.top + nt;
+    m.dtop = m.df + dw;
+    m.n_new = m.dtop + dt;
+    m.list = reinterpret_cast<uint16_t *>(m.n_new + 4);
+    for (uint32_t i = lane; i < nw + nt + dw + dt + 1; i += 32) m.bm[i] = 0u;
+    __syncwarp();
+    const uint64_t *__restrict__ const gcol = D.gcol;
+    const uint4 *__restrict__ const rec = D.rec;
+    const uint32_t *ext2int = reinterpret_cast<const uint32_t *>(arena + L.ext2int_off);
+    uint32_t *const err = reinterpret_cast<uint32_t *>(arena + L.err_off), *const head = err + 1;
+    unsigned char *const base = arena + L.thread_off + (size_t)slot * L.per_thread;
+    uint64_t *const val = reinterpret_cast<uint64_t *>(base), *const regv = val + n_net;
+    uint32_t *const regr = reinterpret_cast<uint32_t *>(regv + 2 * (size_t)L.sreg);
+
+    for (;;) {
+        uint32_t fi = 0;
+        if (lane == 0) fi = atomicAdd(head, 1u);
+        fi = __shfl_sync(FULL, fi, 0);
+        if (fi >= n_faults) return;
+        const StaticFault fx = faults[fi];
+        StaticResult out;
+        uint32_t site = 0;
+        if (!static_site(D, ext2int, fx, err, &out, &site)) {
+            if (lane == 0) results[fi] = out;
+            continue;
+        }
+        const uint64_t bm1 = 1ull << fx.bit;
+        const bool sv = fx.stuck != 0;
+        auto force = [&](uint64_t x) { return sv ? (x | bm1) : (x & ~bm1); };
+        const uint64_t *const scol = gcol + (size_t)site * T;
+        uint32_t nreg = 0, cur = 0, t = 0;
+        while (t < T) {
+            if (nreg == 0) {   // the next cycle in which the fault acts
+                uint32_t hit = 0;
+                for (; t < T; t += 32) {
+                    const bool on = t + lane < T && force(__ldg(scol + min(t + lane, T - 1))) != __ldg(scol + min(t + lane, T - 1));
+                    hit = __ballot_sync(FULL, on);
+                    if (hit) break;
+                }
+                if (!hit) break;
+                t += __ffs((int)hit) - 1;
+            }
+            const uint32_t nb = cur ^ 1u;
+            uint32_t port = NI_NO_PORT;
+            auto mark = [&](uint32_t n) {
+                const uint32_t w = n >> 5;
+                atomicOr(m.bm + w, 1u << (n & 31u));
+                atomicOr(m.top + (w >> 5), 1u << (w & 31u));
+            };
+            // a net that differs: its value, port, latches and consumers (ni: its netinfo)
+            auto keep = [&](uint32_t net, uint64_t v, uint64_t g, uint4 ni, const uint4 *r) {
+                val[net] = v;
+                const uint32_t w = net >> 5;
+                atomicOr(m.df + w, 1u << (net & 31u));
+                atomicOr(m.dtop + (w >> 5), 1u << (w & 31u));
+                port = min(port, ni_port(ni.w));
+                uint32_t nl = ni_nreg(ni.w);
+                if (nl == 255u) nl = D.dreg_off[net + 1] - ni.z;
+                for (uint32_t e = 0; e < nl; ++e) {   // a single one is in the record
+                    const uint32_t rr = nl == 1 ? ni.z : __ldg(D.dreg_rec + ni.z + e);
+                    const uint64_t wm = wmask(rr >> 25);
+                    if ((v & wm) == (g & wm)) continue;
+                    const uint32_t k = atomicAdd(m.n_new, 1u);
+                    regr[nb * L.sreg + k] = rr & 0x1FFFFFFu;
+                    regv[nb * L.sreg + k] = v & wm;
+                }
+                const uint32_t nf = ni.y - ni.x;
+                if (nf <= 8) {
+                    const uint4 e0 = r[2], e1 = r[3];
+                    const uint32_t e[8] = {e0.x, e0.y, e0.z, e0.w, e1.x, e1.y, e1.z, e1.w};
+#pragma unroll
+                    for (uint32_t k = 0; k < 8; ++k)
+                        if (k < nf) mark((e[k] & (PACK_NETS - 1)) - IR);
+                } else {
+                    for (uint32_t e = ni.x; e < ni.y; ++e) mark(__ldg(D.fo_idx + e));
+                }
+            };
+            bool seeded = false;
+            for (uint32_t k = lane; k < nreg; k += 32) {
+                const uint32_t net = I + regr[cur * L.sreg + k];
+                uint64_t qv = regv[cur * L.sreg + k];
+                if (net == site) { qv = force(qv); seeded = true; }
+                const uint64_t g = __ldg(gcol + (size_t)net * T + t);
+                if (qv != g) keep(net, qv, g, __ldg(rec + 8 * (size_t)net + 1), rec + 8 * (size_t)net);
+            }
+            seeded = __any_sync(FULL, seeded);
+            if (lane == 0) {
+                const uint64_t g = __ldg(scol + t);
+                if (force(g) != g) {   // else the site's own evaluation or register decides
+                    if (site >= IR) mark(site - IR);
+                    else if (!seeded) keep(site, force(g), g, __ldg(rec + 8 * (size_t)site + 1), rec + 8 * (size_t)site);
+                }
+            }
+            __syncwarp();
+            uint32_t tp = 0;   // no word of top before it is set
+            for (;;) {
+                uint32_t word = FULL;   // the first word with a dirty node
+                for (; tp < nt; tp += 32) {
+                    const uint32_t x = tp + lane < nt ? m.top[tp + lane] : 0u;
+                    const uint32_t any = __ballot_sync(FULL, x != 0u);
+                    if (!any) continue;
+                    const int src = __ffs((int)any) - 1;
+                    word = (tp + src) * 32 + __ffs((int)__shfl_sync(FULL, x, src)) - 1;
+                    break;
+                }
+                if (word == FULL) break;
+                const uint32_t n0 = word * 32 + __ffs((int)m.bm[word]) - 1;
+                const uint32_t end = __ldg(D.lvl_start + D.node_level[n0] + 1);
+                // its level's dirty nodes in 32 words into the list
+                const uint32_t wi = word + lane;
+                uint32_t bits = 0, at = 0;
+                if (wi < nw && wi * 32 < end) {
+                    const uint32_t all = m.bm[wi];
+                    bits = end - wi * 32 >= 32 ? all : all & ((1u << (end - wi * 32)) - 1u);
+                    if (bits) {
+                        m.bm[wi] = all ^ bits;
+                        if (all == bits) atomicAnd(m.top + (wi >> 5), ~(1u << (wi & 31u)));
+                    }
+                }
+                const uint32_t mine = __popc(bits);
+                uint32_t sum = mine;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t x = __shfl_up_sync(FULL, sum, o);
+                    if (lane >= (uint32_t)o) sum += x;
+                }
+                at = sum - mine;
+                const uint32_t total = __shfl_sync(FULL, sum, 31);
+                for (; bits; bits &= bits - 1) m.list[at++] = (uint16_t)(lane * 32 + __ffs((int)bits) - 1);
+                __syncwarp();
+                for (uint32_t k = lane; k < total; k += 32) {
+                    const uint32_t net = IR + word * 32 + m.list[k];
+                    const uint4 *const r = rec + 8 * (size_t)net;
+                    const uint4 d = __ldg(r), ni = __ldg(r + 1);
+                    const uint64_t g = __ldg(gcol + (size_t)net * T + t);
+                    auto operand = [&](uint32_t x, uint32_t bit) -> uint64_t {
+                        if (!(d.w & bit)) return 0ull;
+                        return m.df[x >> 5] >> (x & 31u) & 1u ? val[x] : __ldg(gcol + (size_t)x * T + t);
+                    };
+                    const uint64_t x = operand(d.x, 1u << 4), y = operand(d.y, 1u << 5), s = operand(d.z, 1u << 6);
+                    uint64_t v = pack_eval(d, x, y, s);
+                    if (net == site) v = force(v);
+                    if (v != g) keep(net, v, g, ni, r);
+                }
+                __syncwarp();
+            }
+            for (uint32_t i = lane; i < dt; i += 32)
+                for (uint32_t x = m.dtop[i]; x; x &= x - 1) m.df[i * 32 + __ffs((int)x) - 1] = 0u;
+            __syncwarp();
+            for (uint32_t i = lane; i < dt; i += 32) m.dtop[i] = 0u;
+            port = __reduce_min_sync(FULL, port);
+            nreg = *(volatile uint32_t *)m.n_new;
+            __syncwarp();
+            if (lane == 0) *m.n_new = 0u;
+            __syncwarp();
+            if (port != NI_NO_PORT) {
+                out.detected = 1;
+                out.cycle = (int32_t)t;
+                out.port = (int32_t)port;
+                break;
+            }
+            cur = nb;
+            ++t;
+        }
+        if (lane == 0) results[fi] = out;
+    }
+}
+
+int static_warps(uint32_t n_node, uint32_t n_net) {
+    const size_t one = static_warp_bytes(n_node, n_net);
+    return (int)std::min<size_t>(4, STATIC_SMEM / one);
+}
+
+cudaError_t launch_static(const DevDesign *d_designs, uint32_t design, uint32_t n_node, uint32_t n_net, const void *faults,
+                          void *results, uint32_t n_faults, uint32_t blocks, uint32_t warps, void *arena, StaticLayout L, cudaStream_t stream) {
+    const size_t smem = warps * static_warp_bytes(n_node, n_net);
+    cudaError_t e = cudaFuncSetAttribute(static_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    static_kernel<<<blocks, warps * 32, smem, stream>>>(d_designs, design, (const StaticFault *)faults, (StaticResult *)results,
+                                                        n_faults, (unsigned char *)arena, L);
+    return cudaGetLastError();
+}
+
+// The form for designs whose bitmaps do not fit in a warp's shared memory (static_warps is 0).
 // One thread per fault of this wave; the wave's scratch is carved from the static array:
 // [ext2int: n_net u32][error word][per thread: values u64, stamps u32, queued u32, heap u32,
 // register diffs 2 x (u32 reg, u64 value)]. Stamps must be zero before the wave.
@@ -101,20 +304,8 @@ plain_static_kernel(const DevDesign *__restrict__ designs, uint32_t design,
 
     const StaticFault fx = faults[fi];
     StaticResult out;
-    out.cycle = -1;
-    out.port = -1;
-    out.detected = 0;
-    out.reserved[0] = out.reserved[1] = out.reserved[2] = 0;
-    if (fx.net >= D.n_net || fx.stuck > 1) {
-        atomicOr(err, 1u);
-        out.detected = 254;
-        results[fi] = out;
-        return;
-    }
-    const uint32_t site = ext2int[fx.net];
-    if (fx.bit >= D.net_w[site]) {
-        atomicOr(err, 1u);
-        out.detected = 254;
+    uint32_t site = 0;
+    if (!static_site(D, ext2int, fx, err, &out, &site)) {
         results[fi] = out;
         return;
     }
@@ -161,7 +352,7 @@ plain_static_kernel(const DevDesign *__restrict__ designs, uint32_t design,
             for (uint32_t e = D.fo_off[net]; e < D.fo_off[net + 1]; ++e) push(D.fo_idx[e]);
             for (uint32_t e = D.dreg_off[net]; e < D.dreg_off[net + 1]; ++e) {
                 const uint32_t r = D.dreg_idx[e];
-                const uint64_t wm = s_wmask(D.net_w[I + r]);
+                const uint64_t wm = wmask(D.net_w[I + r]);
                 if ((v & wm) != (g & wm)) {
                     regr[nb * L.sreg + nreg_new] = r;
                     regv[nb * L.sreg + nreg_new] = v & wm;
@@ -189,13 +380,13 @@ plain_static_kernel(const DevDesign *__restrict__ designs, uint32_t design,
         while (nh > 0) {
             const uint32_t n = pop();
             const uint4 d = D.desc[n];
-            const int no = s_nops(meta_op(d.w));
+            const int no = n_operands(meta_op(d.w));
             uint64_t a = 0, b = 0, c = 0;
             if (no >= 1) a = lookup(d.x);
             if (no >= 2) b = lookup(d.y);
             if (no >= 3) c = lookup(d.z);
             const uint32_t net = IR + n;
-            uint64_t v = s_eval(d, a, b, c);
+            uint64_t v = eval_op(d, a, b, c);
             if (net == site) v = force(v);
             const uint64_t g = gcol[(size_t)net * T + t];
             if (v != g) keep(net, v, g);
