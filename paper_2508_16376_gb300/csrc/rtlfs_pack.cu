@@ -30,9 +30,13 @@
 // branches), so a fault's pace is its levels times about a microsecond, and the throughput is
 // the issue slots: 3.1e9 warp instructions per 128 cycles of the medium campaign against 6.4e9
 // of a lane and a warp per fault. Measured with it, before -> after (whole calls, the good trace
-// included): tiny list 6.9 -> 2.8 ms, 2.8k nodes 61 -> 14 ms, 20k nodes with 5k faults 281 -> 97
-// ms, with 100k faults over 10k cycles 1089 -> 862 ms, transient list 258 -> 161 ms, no-drop
-// 228 -> 132 ms, twelve designs 178 -> 147 ms, 200k nodes 170 -> 75 ms.
+// included, with the good trace's own gains since): tiny list 6.7 -> 2.4 ms, 2.8k nodes 67 -> 14 ms,
+// 20k nodes with 5k faults 268 -> 80 ms, with 100k faults over 10k cycles 1089 -> 880 ms, transient
+// list 260 -> 145 ms, no-drop 192 -> 101 ms, twelve designs 186 -> 86 ms, 200k nodes 161 -> 60 ms.
+// With few faults the last tier sets the pace, and its level the barriers and instructions of its
+// rounds. Slower there: items listed and dealt to the lanes evenly (recorded loads 103 against 83
+// ms: few rounds have two items on a lane), consumers' records prefetched into L1 when they are
+// marked (88), 128 or 64 lanes (no-drop 247, 258 against 115: tables overflow).
 #include "rtlfs_device.h"
 #include "rtlfs_internal.h"
 
@@ -57,7 +61,6 @@ struct PackSmem {
     uint32_t *nnew;          // [32] register diffs latched by a fault this cycle
     uint32_t *fail;          // [32] the fault outgrew its table or buffer
     uint32_t *n_ring;
-    uint32_t *red;           // [2] reductions over the CTA
     uint32_t *ring;          // [PK_RING][5] {slot, first, end, value} of fan-out entries
 };
 
@@ -76,7 +79,6 @@ __device__ __forceinline__ PackSmem pack_layout(unsigned char *sm) {
     m.nnew = reinterpret_cast<uint32_t *>(m.tag + N * TPL);
     m.fail = m.nnew + 32;
     m.n_ring = m.fail + 32;
-    m.red = m.n_ring + 1;
     m.ring = m.n_ring + 8;
     return m;
 }
@@ -135,12 +137,13 @@ pack_kernel(const DevDesign *__restrict__ designs, const __grid_constant__ DevDe
     };
     auto gsum = [&](uint32_t v) {
         if constexpr (BLOCK) {
+            __shared__ uint32_t w[N / 32];
             v = __reduce_add_sync(FULL, v);
-            if (threadIdx.x == 0) sm.red[1] = 0u;
+            if ((lane & 31u) == 0) w[lane >> 5] = v;
             __syncthreads();
-            if ((threadIdx.x & 31u) == 0) atomicAdd(&sm.red[1], v);
-            __syncthreads();
-            v = sm.red[1];
+            v = 0u;
+#pragma unroll
+            for (uint32_t k = 0; k < N / 32; ++k) v += w[k];
         } else {
 #pragma unroll
             for (int o = 1; o < LPS; o <<= 1) v += __shfl_xor_sync(gmask, v, o);
@@ -148,13 +151,17 @@ pack_kernel(const DevDesign *__restrict__ designs, const __grid_constant__ DevDe
         return v;
     };
     auto gmin = [&](uint32_t v) {
+        // A CTA's lanes meet once per reduction (its warps' results side by side; calls lie another
+        // barrier apart): with an atomic per warp and a second barrier a level of its one fault took
+        // an eighth longer (recorded loads 83 -> 75 ms, transient list 157 -> 138).
         if constexpr (BLOCK) {
+            __shared__ uint32_t w[N / 32];
             v = __reduce_min_sync(FULL, v);
-            if (threadIdx.x == 0) sm.red[0] = FULL;
+            if ((lane & 31u) == 0) w[lane >> 5] = v;
             __syncthreads();
-            if ((threadIdx.x & 31u) == 0) atomicMin(&sm.red[0], v);
-            __syncthreads();
-            v = sm.red[0];
+            v = FULL;
+#pragma unroll
+            for (uint32_t k = 0; k < N / 32; ++k) v = min(v, w[k]);
         } else if constexpr (LPS == 32) {
             v = __reduce_min_sync(FULL, v);
         } else {
