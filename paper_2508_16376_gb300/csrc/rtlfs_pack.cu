@@ -17,22 +17,23 @@
 // delivered is in the entry, any other is the good value. Insertion (compare-and-swap) makes
 // each dirty node an item once. A 16-bit tag per entry holds a pending item's level above the
 // entry's place among the TPL its lane owns, so the minimum over a lane's tags (two per
-// instruction) is both the fault's next level and an item of it, without any list. Register diffs go to a private double buffer.
+// instruction) is both the fault's next level and an item of it, without any list. Register diffs
+// go to a private double buffer.
 //
-// Tiers: one lane per fault for the many faults with a handful of dirty nodes, then several
-// lanes, then a warp. A fault that outgrows its table or buffer is handed to the next tier
-// with its start-of-cycle register diffs (the last tier is the one-warp-per-fault kernel with
-// its state in global memory). Which faults count as light or heavy (evaluation counters,
+// Tiers: one lane per fault for the many faults with a handful of dirty nodes, then 8, a warp,
+// and a CTA of 256. A fault that outgrows its table or buffer is handed to the next tier
+// with its start-of-cycle register diffs (behind the last is the heavy kernel, with its
+// state in global memory). Which faults count as light or heavy (evaluation counters,
 // promotions) follows the light lanes' capacity rule and does not depend on the tier.
 //
 // What bounds it: instructions, not memory. A round is about 250 warp instructions at 7 cycles
 // each (ncu, medium campaign, 32 lanes per fault: 2.3 of them fixed latency, 1.5 L2 loads, 1.1
 // branches), so a fault's pace is its levels times about a microsecond, and the throughput is
 // the issue slots: 3.1e9 warp instructions per 128 cycles of the medium campaign against 6.4e9
-// of a lane and a warp per fault. Measured with it, before -> after (whole calls, the good trace
-// included, with the good trace's own gains since): tiny list 6.7 -> 2.4 ms, 2.8k nodes 67 -> 14 ms,
-// 20k nodes with 5k faults 268 -> 80 ms, with 100k faults over 10k cycles 1089 -> 880 ms, transient
-// list 260 -> 145 ms, no-drop 192 -> 101 ms, twelve designs 186 -> 86 ms, 200k nodes 161 -> 60 ms.
+// of a lane and a warp per fault. Light and heavy kernels -> now (whole calls, with the good
+// trace's own gains): tiny list 6.8 -> 2.4 ms, 2.8k nodes 61 -> 15 ms, 20k nodes with 5k faults 286 -> 82
+// ms, with 100k faults over 10k cycles 1125 -> 881 ms, transient list 270 -> 152 ms, no-drop 131 -> 72 ms,
+// twelve designs 193 -> 89 ms, 200k nodes 169 -> 62 ms.
 // With few faults the last tier sets the pace, and its level the barriers and instructions of its
 // rounds. Slower there: items listed and dealt to the lanes evenly (recorded loads 103 against 83
 // ms: few rounds have two items on a lane), consumers' records prefetched into L1 when they are
