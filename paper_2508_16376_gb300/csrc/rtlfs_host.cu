@@ -1257,22 +1257,24 @@ int take_checkpoint(rtlfs_ctx *ctx, uint32_t nw, uint32_t w_end, uint32_t W, uin
             c.pool_v.insert(c.pool_v.end(), pv.begin(), pv.end());
         }
         // sorted as the light and heavy kernels leave them: light faults (at most the light
-        // capacity's register diffs) with their state in st_*, heavy ones in the pool
+        // capacity's register diffs) with their state in st_*, heavy ones in the pool, and with
+        // them any whose register diffs st_* and its byte-sized count do not hold
+        const uint32_t cap = (uint32_t)LIGHT_CAPS[lcap][0];
         std::vector<uint8_t> cls;
         if ((r = get(cls, ctx->pk_cls.p, F))) return r;
         std::vector<uint32_t> light;
         std::vector<HeavyCarry> heavy;
         for (const HeavyCarry &x : c.carry) {
-            if (cls[x.fault]) { heavy.push_back(x); continue; }
+            if (cls[x.fault] || x.nreg > cap) { heavy.push_back(x); continue; }
             light.push_back(x.fault);
             c.st_nreg[x.fault] = (uint8_t)x.nreg;
-            for (uint32_t k = 0; k < x.nreg && k < (uint32_t)LIGHT_KR; ++k) {
+            for (uint32_t k = 0; k < x.nreg; ++k) {
                 c.st_r[(size_t)k * F + x.fault] = c.pool_r[x.off + k];
                 c.st_v[(size_t)k * F + x.fault] = c.pool_v[x.off + k];
             }
         }
         for (uint32_t x : c.live) {
-            if (!cls[x]) { light.push_back(x); continue; }
+            if (!cls[x] && c.st_nreg[x] <= cap) { light.push_back(x); continue; }
             heavy.push_back(HeavyCarry{x, c.st_nreg[x], c.pool_r.size()});
             for (uint32_t k = 0; k < c.st_nreg[x]; ++k) {
                 c.pool_r.push_back(c.st_r[(size_t)k * F + x]);

@@ -383,16 +383,19 @@ pack_kernel(const DevDesign *__restrict__ designs, const __grid_constant__ DevDe
                 if (active) {
                     const uint32_t ev = gsum(my_ev), nr = sm.nnew[slot];
                     port = gmin(my_port);
-                    if (sm.fail[slot]) {
+                    // the capacity rule: more register diffs or evaluations in a cycle than a light
+                    // fault may have make the fault heavy, that cycle included; so does a cycle
+                    // that not even the last tier holds (its table and buffer are far beyond the
+                    // rule), which the heavy kernel simulates without looking at the class
+                    const bool full = sm.fail[slot] != 0u;
+                    if (!heavy && (full ? BLOCK : nr > q.cap_regs || ev > q.cap_evals)) {
+                        heavy = true;
+                        t_heavy = t;
+                        if (sub == 0) atomicAdd(q.prom_total, 1u);
+                    }
+                    if (full) {
                         next = PROMOTE;
                     } else {
-                        // the light lanes' capacity rule: more register diffs or evaluations in
-                        // a cycle than a lane holds make the fault heavy, that cycle included
-                        if (!heavy && (nr > q.cap_regs || ev > q.cap_evals)) {
-                            heavy = true;
-                            t_heavy = t;
-                            if (sub == 0) atomicAdd(q.prom_total, 1u);
-                        }
                         (heavy ? ev_heavy : ev_light) += ev;
                         if (port != NI_NO_PORT && detect(port)) {
                             next = DETECTED;
