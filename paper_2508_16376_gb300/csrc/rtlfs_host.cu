@@ -1764,10 +1764,12 @@ static int run_campaign(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_res
             int r4 = restore_checkpoint(ctx, nw, w_begin, prom_total);
             if (r4 != RTLFS_OK) return r4;
             if (pk.use && F) {   // the carried faults count as heavy
+                // on the stream whose event the kernels wait for: a plain copy is ordered only
+                // with the legacy stream, which theirs do not wait for
                 std::vector<uint8_t> cls(F, 0);
                 for (const HeavyCarry &x : ctx->ck.carry) cls[x.fault] = 1;
-                CU(cudaStreamSynchronize(ctx->s_main));
-                CU(cudaMemcpy(ctx->pk_cls.p, cls.data(), F, cudaMemcpyHostToDevice));
+                CU(cudaMemcpyAsync(ctx->pk_cls.p, cls.data(), F, cudaMemcpyHostToDevice, ctx->s_main));
+                CU(cudaStreamSynchronize(ctx->s_main));   // cls is gone at the end of this block
             }
         }
         CU(cudaEventRecord(ctx->ev_wl, ctx->s_main));
