@@ -916,8 +916,17 @@ int launch_good(rtlfs_ctx *ctx, uint32_t *n_launches = nullptr) {
     return RTLFS_OK;
 }
 
+// Host-to-device copies go through the legacy stream; one from pageable memory may return before
+// it has landed, and the context's (non-blocking) streams do not wait for that stream. Every call
+// that launches on them after such copies comes through here first.
+int uploads_landed(rtlfs_ctx *ctx) {
+    CU(cudaStreamSynchronize(cudaStreamLegacy));
+    return RTLFS_OK;
+}
+
 int enqueue_good(rtlfs_ctx *ctx) {
     int rc = prepare_good(ctx);
+    if (rc == RTLFS_OK) rc = uploads_landed(ctx);
     return rc != RTLFS_OK ? rc : launch_good(ctx);
 }
 
@@ -2036,6 +2045,8 @@ static int run_campaign(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_res
         return RTLFS_OK;
     };
 
+    rc = uploads_landed(ctx);
+    if (rc != RTLFS_OK) return rc;
     if (o.use_graph) {
         // Everything the captured work depends on by address or size.
         std::vector<uint64_t> key = {F, n_heavy, ql.n_light, (uint64_t)lcap, (uint64_t)lblock,
@@ -2326,6 +2337,7 @@ int rtlfs_features(rtlfs_ctx *ctx, uint32_t design_id, float *out) {
         if (!D->trace_valid) { rc = run_good_only(ctx); if (rc != RTLFS_OK) return rc; break; }
     if (!ctx->F) return RTLFS_OK;
     rc = ensure_sched_buffers(ctx);
+    if (rc == RTLFS_OK) rc = uploads_landed(ctx);
     if (rc != RTLFS_OK) return rc;
     CU(launch_features(ctx->d_designs.p, dev_faults(ctx), ctx->d_static_ptrs.p, ctx->d_X.p,
                        ctx->d_heur.p, ctx->s_main));
@@ -2373,7 +2385,7 @@ static int upload_samples(rtlfs_ctx *ctx, const float *X, const float *t, uint32
         CU(ctx->d_ty.reserve(n));
         CU(cudaMemcpy(ctx->d_ty.p, t, (size_t)n * sizeof(float), cudaMemcpyHostToDevice));
     }
-    return RTLFS_OK;
+    return uploads_landed(ctx);
 }
 
 int rtlfs_mlp_forward(rtlfs_ctx *ctx, const float *X, uint32_t n, float *y) {
