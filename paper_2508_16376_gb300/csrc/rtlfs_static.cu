@@ -201,13 +201,14 @@ static_kernel(const DevDesign *__restrict__ designs, uint32_t design, const Stat
                     break;
                 }
                 if (word == FULL) break;
-                const uint32_t n0 = word * 32 + __ffs((int)m.bm[word]) - 1;
-                const uint32_t end = __ldg(D.lvl_start + D.node_level[n0] + 1);
-                // its level's dirty nodes in 32 words into the list
+                // its level's dirty nodes in 32 words into the list: each lane reads and clears a word
+                // of its own, and the first lane's, which names the level, comes by a shuffle
                 const uint32_t wi = word + lane;
+                const uint32_t all = wi < nw ? m.bm[wi] : 0u;
+                const uint32_t n0 = word * 32 + __ffs((int)__shfl_sync(FULL, all, 0)) - 1;
+                const uint32_t end = __ldg(D.lvl_start + D.node_level[n0] + 1);
                 uint32_t bits = 0, at = 0;
                 if (wi < nw && wi * 32 < end) {
-                    const uint32_t all = m.bm[wi];
                     bits = end - wi * 32 >= 32 ? all : all & ((1u << (end - wi * 32)) - 1u);
                     if (bits) {
                         m.bm[wi] = all ^ bits;
