@@ -728,7 +728,9 @@ int build_cluster_plan(rtlfs_ctx *ctx, Design &D, uint32_t C, int lc) {
         return (reg ? CL_REG : 0u) | (k == me ? CL_SELF : 0u) | (k << CL_RANK_SHIFT) | (reg ? P->own + reg_at[net - I] : slot[net - IR]);
     };
     const size_t per_cta = (size_t)P->steps * width;
-    std::vector<uint4> cdesc(C * per_cta + 1, make_uint4(0, 0, 0, 0));
+    // a blank record behind the last, and, in a design without nodes, those of the two steps that a
+    // thread reads ahead
+    std::vector<uint4> cdesc(std::max<size_t>(C * per_cta + 1, 2 * width), make_uint4(0, 0, 0, 0));
     std::vector<std::vector<uint4>> consts(C);
     for (auto &u : used) std::fill(u.begin(), u.end(), 0u);
     for (uint32_t n = 0; n < N; ++n) {   // in node order within a step: neighbours share trace lines

@@ -79,7 +79,7 @@ struct DevDesign {
     uint32_t cl_steps;          // steps of a cycle, an even number
     uint32_t cl_width;          // nodes a CTA evaluates per step, at most (a multiple of 32)
     uint32_t cl_latch_sync;     // some register's D net is a node of another CTA
-    const uint4    *cl_desc;    // [C][cl_steps][cl_width] records, and a blank one
+    const uint4    *cl_desc;    // [C][cl_steps][cl_width] records, and a blank one (2 cl_width blank ones when there are no steps)
     const uint4    *cl_reg;     // {register, D location, width, D net} by home CTA
     const uint32_t *cl_reg_off; // [C + 1] registers of each CTA
     const uint4    *cl_const;   // {slot, value lo, hi, 0}: constant nodes by CTA
