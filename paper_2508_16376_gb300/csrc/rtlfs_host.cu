@@ -1811,6 +1811,9 @@ static int run_campaign(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_res
         }
         for (uint32_t w = w_begin; w < w_end; ++w) {
             const uint32_t t0 = w * W, t1 = std::min(t0 + W, Tmax);
+            // a window that the packed form made inside the caller's (or inside the one pass)
+            // shows nowhere, so not in when the budget stops a fault either
+            const bool budget_at_end = W != WU && (WU == 0 || t1 % WU != 0);
             // good trace of the window (and of the windows the scheduler needs)
             for (; g_next <= std::max(w, w_sched ? w_sched - 1 : 0u) && g_next < nw; ++g_next) {
                 const uint32_t g0 = g_next * W, g1 = std::min(g0 + W, Tmax);
@@ -1865,6 +1868,7 @@ static int run_campaign(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_res
                 // behind the last): each takes what the tier before handed on in this window
                 PackArgs pa = pack_args();
                 pa.t0 = t0; pa.t1 = t1;
+                pa.budget_at_end = budget_at_end;
                 pa.prom_total = prom_total;
                 pa.prom_top = pk64 + 2 * PT * nw;
                 const int in = w & 1 ? 0 : 1, out = w & 1;   // window parity of the ping-pong buffers
@@ -1945,6 +1949,7 @@ static int run_campaign(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_res
             wh.t1 = t1;
             wh.budget_hit = ctx->d_heads.p + 3;
             wh.fault_budget = o.fault_budget;
+            wh.budget_at_end = budget_at_end;
             wh.counters = ctx->d_heads.p + 6;
             wh.err = ctx->d_err.p;
             if (pk.use) {   // the faults the last tier handed on, to the end of the window only:
@@ -2053,7 +2058,7 @@ static int run_campaign(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_res
         // Everything the captured work depends on by address or size.
         std::vector<uint64_t> key = {F, n_heavy, ql.n_light, (uint64_t)lcap, (uint64_t)lblock,
                                      (uint64_t)lgrid, (uint64_t)hblock, (uint64_t)hgrid,
-                                     (uint64_t)dev_sched, (uint64_t)use_mlp, o.fault_budget, W,
+                                     (uint64_t)dev_sched, (uint64_t)use_mlp, o.fault_budget, W, WU,
                                      (uint64_t)nodrop, (uint64_t)good_first, (uint64_t)o.order_classes,
                                      (uint64_t)pk.use, (uint64_t)pk.grid};
         const void *ptrs[] = {ctx->d_designs.p, ctx->d_list_smem.p, ctx->d_list_glob.p, ctx->d_order.p, ctx->d_err.p, ctx->h_gbm.p,

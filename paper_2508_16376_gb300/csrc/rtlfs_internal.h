@@ -254,6 +254,7 @@ struct WinHeavy {
     uint32_t t0, t1;
     unsigned long long *budget_hit;
     uint64_t fault_budget;
+    uint32_t budget_at_end;       // as in PackArgs
     unsigned long long *counters;
     uint32_t *err;                // bit 1: pool overflow
 };
@@ -306,6 +307,7 @@ struct PackArgs {
     uint32_t *prom_total;         // light faults that became heavy
     unsigned long long *budget_hit;
     uint64_t fault_budget;
+    uint32_t budget_at_end;       // the window's end is not one of the caller's: the budget holds there too
     unsigned long long *counters_light, *counters_heavy;   // [0] evaluations, [1] fault-cycles
     uint32_t *err;                // bit 1: pool overflow
 };

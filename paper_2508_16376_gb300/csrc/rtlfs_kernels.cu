@@ -776,6 +776,7 @@ struct HeavyRun {
     int status;        // 0 alive at tend, 1 detected at t, 3 over the load budget
     int32_t det_cycle, det_port;
     uint32_t mism;     // no-drop mode: cycles of this run with a differing output
+    bool budget_at_end;   // in: the budget holds after cycle tend - 1 too
 };
 
 // Simulate fault fid from cycle r.t until it is detected, exceeds the load budget or
@@ -927,8 +928,9 @@ __device__ __forceinline__ void heavy_run_fault(const DevDesign &D, const DevFau
                 if (tid == 0) V.load += 1;
                 if (detect(fs.port)) break;
                 __syncthreads();
-                if (++t >= tend) break;
+                if (++t >= tend && !r.budget_at_end) break;
                 if (budget && (f.load[fid] + V.load) > budget) { status = 3; break; }
+                if (t >= tend) break;
                 continue;
             }
         }
@@ -1067,8 +1069,9 @@ __device__ __forceinline__ void heavy_run_fault(const DevDesign &D, const DevFau
         if (V.minport != NI_NO_PORT && detect(V.minport)) break;
         nreg = V.nreg_new;
         cur = nb;
-        if (++t >= tend) break;
+        if (++t >= tend && !r.budget_at_end) break;
         if (budget && (f.load[fid] + V.load) > budget) { status = 3; break; }
+        if (t >= tend) break;
         __syncthreads();
     }
     r.t = t;
@@ -1225,8 +1228,9 @@ __device__ __forceinline__ void heavy_run_fault_warp(const DevDesign &D, const D
                 // a port fault changes only what its port observes of the site net
                 ++load;
                 if (detect(fs.port)) break;
-                if (++t >= tend) break;
+                if (++t >= tend && !r.budget_at_end) break;
                 if ((long long)load > room) { status = 3; break; }
+                if (t >= tend) break;
                 continue;
             }
         }
@@ -1400,8 +1404,9 @@ __device__ __forceinline__ void heavy_run_fault_warp(const DevDesign &D, const D
         if (minport != NI_NO_PORT && detect(minport)) break;
         nreg = V.nreg_new;
         cur = nb;
-        if (++t >= tend) break;
+        if (++t >= tend && !r.budget_at_end) break;
         if ((long long)load > room) { status = 3; break; }
+        if (t >= tend) break;
         __syncwarp();
     }
     __syncwarp();
@@ -1523,7 +1528,7 @@ heavy_window_kernel(const DevDesign *__restrict__ designs, DevFaults f, WinHeavy
         }
         if (tid == 0) V.load = 0;
         hsync<WARP>();
-        HeavyRun r{t_start, nreg0, 0, 0, -1, -1, 0};
+        HeavyRun r{t_start, nreg0, 0, 0, -1, -1, 0, q.budget_at_end && tend < D.T};
         if (WARP) heavy_run_fault_warp<EXACT, GBM>(D, f, fid, tend, q.fault_budget, sm, V, fval, stamp, regR, regV, S.max_reg, S.max_net, r);
         else heavy_run_fault<EXACT>(D, f, fid, tend, q.fault_budget, sm, V, fval, stamp, regR, regV, S.max_reg, S.max_net, r);
         hsync<WARP>();

@@ -317,7 +317,10 @@ pack_kernel(const DevDesign *__restrict__ designs, const __grid_constant__ DevDe
         ++mism;
         return false;
     };
-    auto over_budget = [&]() -> bool { return q.fault_budget && before + ev_light + ev_heavy > q.fault_budget; };
+    // after a completed cycle, before cycle t; not at the end of one of the caller's windows
+    auto over_budget = [&]() -> bool {
+        return q.fault_budget && before + ev_light + ev_heavy > q.fault_budget && (t < tend || (q.budget_at_end && t < cycles()));
+    };
     // What becomes of the fault at cycle t.
     enum { RUN, DETECTED, BUDGET, END, PROMOTE };
     uint32_t port = NI_NO_PORT;   // the detecting port
@@ -344,7 +347,7 @@ pack_kernel(const DevDesign *__restrict__ designs, const __grid_constant__ DevDe
             port = fs.port;
             if (detect(port)) return DETECTED;
             ++t;
-            if (t < tend && over_budget()) return BUDGET;
+            if (over_budget()) return BUDGET;
         }
     };
 
@@ -403,7 +406,7 @@ pack_kernel(const DevDesign *__restrict__ designs, const __grid_constant__ DevDe
                             cur ^= 1u;
                             nreg = nr;
                             ++t;
-                            if (t < tend && over_budget()) next = BUDGET;
+                            if (over_budget()) next = BUDGET;
                             else if (t < tend && ev > q.tier_evals) next = PROMOTE;   // slow here
                         }
                     }
