@@ -114,6 +114,37 @@ struct GoodLaunch {
 // Kernels of a window that are timed: light and heavy, or the packed tiers and the heavy kernel.
 constexpr size_t WIN_TIMED = PACK_TIERS + 1;
 
+// Scratch and form of a launch of the heavy kernel: a slot per CTA.
+struct HeavySet {
+    DBuf<HeavyVal> fval;
+    DBuf<uint32_t> stamp;
+    DBuf<uint32_t> regr;
+    DBuf<uint64_t> regv;
+    DBuf<uint32_t> gbm;
+    uint32_t slots = 0, grid = 0, max_net = 0, max_reg = 0, max_node = 0, max_levels = 0;
+    bool exact = false;                // the form for the current designs
+    bool use_gbm = false;              // node bitmaps in global scratch (gbm)
+    bool stamps_stale = false;         // the exact form wrote values over stamp fields since
+
+    HeavyScratch view() const {
+        HeavyScratch v{};
+        v.fval = fval.p;
+        v.stamp = stamp.p;
+        v.reg_r = regr.p; v.reg_v = regv.p;
+        v.max_net = max_net; v.max_reg = max_reg; v.max_node = max_node;
+        v.exact = exact ? 1u : 0u;
+        v.gbm = use_gbm ? gbm.p : nullptr;
+        v.max_levels = max_levels;
+        return v;
+    }
+    // what a captured launch depends on
+    void add_key(std::vector<uint64_t> &key) const {
+        key.insert(key.end(), {(uint64_t)(uintptr_t)fval.p, (uint64_t)(uintptr_t)stamp.p, (uint64_t)(uintptr_t)regr.p,
+                               (uint64_t)(uintptr_t)regv.p, (uint64_t)(uintptr_t)gbm.p, grid, max_net, max_reg, max_node,
+                               max_levels, (uint64_t)exact, (uint64_t)use_gbm});
+    }
+};
+
 struct rtlfs_ctx {
     int device = 0;
     GoodLaunch gl;
@@ -178,15 +209,7 @@ struct rtlfs_ctx {
                                       // bit 2: a cluster good-trace launch ran without its clusters
     DBuf<unsigned long long> d_heads; // [0] light, [1] init heavy, [2] prom heavy, [3] budget,
                                       // [4..5] light evals/cycles, [6..7] heavy evals/cycles
-    DBuf<HeavyVal> h_fval;
-    DBuf<uint32_t> h_stamp;
-    DBuf<uint32_t> h_regr;
-    DBuf<uint64_t> h_regv;
-    uint32_t heavy_slots = 0, heavy_grid = 0, hs_net = 0, hs_reg = 0, hs_node = 0, hs_lv = 0;
-    bool heavy_exact = false;          // the heavy kernel's form for the current designs
-    bool heavy_gbm = false;            // node bitmaps in global scratch (h_gbm)
-    DBuf<uint32_t> h_gbm;
-    bool stamps_stale = false;         // the exact form wrote values over stamp fields since
+    HeavySet heavy, crowd;             // the heavy kernel's, and the one for the packed form's crowds
                                        // the scratch was last zeroed
     // scheduler state
     DBuf<const float *> d_static_ptrs;
@@ -989,7 +1012,7 @@ DevFaults dev_faults(rtlfs_ctx *ctx) {
     return f;
 }
 
-int ensure_heavy_scratch(rtlfs_ctx *ctx, int block, int want_slots, int form) {
+int ensure_heavy_scratch(rtlfs_ctx *ctx, HeavySet &h, int block, int want_slots, int form) {
     uint32_t mn = 1, mr = 1, mnode = 1, ml = 1;
     for (Design *D : ctx->designs) {
         mn = std::max(mn, D->n_net); mr = std::max(mr, D->R);
@@ -1015,53 +1038,41 @@ int ensure_heavy_scratch(rtlfs_ctx *ctx, int block, int want_slots, int form) {
     }
     const int per_sm = gbm ? per_sm_g : exact ? per_sm_x : per_sm_s;
     if (per_sm < 1) return fail(ctx, RTLFS_E_ARG, "heavy kernel cannot be resident with block %d", block);
-    ctx->heavy_exact = exact;
-    ctx->heavy_gbm = gbm;
+    h.exact = exact;
+    h.use_gbm = gbm;
     if (exact) {
-        ctx->stamps_stale = true;   // its 8-byte values overwrite stamp fields
+        h.stamps_stale = true;   // its 8-byte values overwrite stamp fields
     }
     int slots = want_slots > 0 ? want_slots : per_sm * ctx->n_sm;
     slots = std::min(slots, per_sm * ctx->n_sm);
-    const bool grow = slots > (int)ctx->heavy_slots || mn > ctx->hs_net || mr > ctx->hs_reg;
+    const bool grow = slots > (int)h.slots || mn > h.max_net || mr > h.max_reg;
     if (grow) {
-        ctx->h_fval.release(); ctx->h_regr.release(); ctx->h_regv.release(); ctx->h_stamp.release();
-        CU(ctx->h_fval.reserve((size_t)slots * mn));
-        CU(ctx->h_stamp.reserve((size_t)slots));
-        ctx->stamps_stale = true;   // fresh memory: zeroed below before a stamped run
-        CU(ctx->h_regr.reserve((size_t)slots * 2 * mr));
-        CU(ctx->h_regv.reserve((size_t)slots * 2 * mr));
-        ctx->heavy_slots = slots; ctx->hs_net = mn; ctx->hs_reg = mr;
+        h.fval.release(); h.regr.release(); h.regv.release(); h.stamp.release();
+        CU(h.fval.reserve((size_t)slots * mn));
+        CU(h.stamp.reserve((size_t)slots));
+        h.stamps_stale = true;   // fresh memory: zeroed below before a stamped run
+        CU(h.regr.reserve((size_t)slots * 2 * mr));
+        CU(h.regv.reserve((size_t)slots * 2 * mr));
+        h.slots = slots; h.max_net = mn; h.max_reg = mr;
     }
-    ctx->hs_node = mnode; ctx->hs_lv = ml;
-    ctx->heavy_grid = (uint32_t)slots;
+    h.max_node = mnode; h.max_levels = ml;
+    h.grid = (uint32_t)slots;
     if (gbm) {   // node bitmaps start zero and every fault leaves them zero
         const size_t need = (size_t)slots * ((mnode + 31) / 32);
-        if (ctx->h_gbm.n < need) {
-            ctx->h_gbm.release();
-            CU(ctx->h_gbm.reserve(need));
-            CU(cudaMemsetAsync(ctx->h_gbm.p, 0, ctx->h_gbm.n * sizeof(uint32_t), ctx->s_main));
+        if (h.gbm.n < need) {
+            h.gbm.release();
+            CU(h.gbm.reserve(need));
+            CU(cudaMemsetAsync(h.gbm.p, 0, h.gbm.n * sizeof(uint32_t), ctx->s_main));
         }
     }
-    if (!exact && ctx->stamps_stale) {
+    if (!exact && h.stamps_stale) {
         // stamp 0 is never current: zeroed entries and counters start every slot clean
         // (on the main stream, which every heavy launch of the campaign waits behind)
-        CU(cudaMemsetAsync(ctx->h_fval.p, 0, ctx->h_fval.n * sizeof(HeavyVal), ctx->s_main));
-        CU(cudaMemsetAsync(ctx->h_stamp.p, 0, ctx->h_stamp.n * sizeof(uint32_t), ctx->s_main));
-        ctx->stamps_stale = false;
+        CU(cudaMemsetAsync(h.fval.p, 0, h.fval.n * sizeof(HeavyVal), ctx->s_main));
+        CU(cudaMemsetAsync(h.stamp.p, 0, h.stamp.n * sizeof(uint32_t), ctx->s_main));
+        h.stamps_stale = false;
     }
     return RTLFS_OK;
-}
-
-HeavyScratch heavy_view(rtlfs_ctx *ctx) {
-    HeavyScratch s{};
-    s.fval = ctx->h_fval.p;
-    s.stamp = ctx->h_stamp.p;
-    s.reg_r = ctx->h_regr.p; s.reg_v = ctx->h_regv.p;
-    s.max_net = ctx->hs_net; s.max_reg = ctx->hs_reg; s.max_node = ctx->hs_node;
-    s.exact = ctx->heavy_exact ? 1u : 0u;
-    s.gbm = ctx->heavy_gbm ? ctx->h_gbm.p : nullptr;
-    s.max_levels = ctx->hs_lv;
-    return s;
 }
 
 // The packed faulty-machine form for the loaded designs.
@@ -1070,6 +1081,7 @@ struct PackPlan {
     int grid = 0;
     int warps[PACK_TIERS] = {};
     uint32_t evals[PACK_TIERS] = {};   // evaluations in a cycle beyond which a fault moves on
+    uint32_t limit[PACK_TIERS] = {};   // faults beyond which a tier hands all of them on
 };
 
 // The packed form runs whenever its tags can name the levels of every design and 27 bits its
@@ -1086,10 +1098,22 @@ PackPlan plan_pack(rtlfs_ctx *ctx, int heavy_form) {
     // what a tier handles in a few rounds, and the tiers' shares of an SM follow their work.
     // (medium campaign, 658 faults per SM, windows of 128: 922 against 1402 ms; transient list,
     // 197 per SM, windows of 256: 199 against 182)
-    const bool many = ctx->F > 400u * (uint32_t)ctx->n_sm;
+    bool narrow = true;   // levels narrower than four warps: a CTA has little over a warp
+    for (Design *D : ctx->designs) narrow = narrow && D->N <= 128ull * D->n_levels;
+    const uint64_t sms = (uint64_t)ctx->n_sm;
+    const bool many = ctx->F > 400u * sms;
     const int w[2][PACK_TIERS] = {{5, 4, 4, 1}, {3, 5, 7, 1}};
     const uint32_t e[2][PACK_TIERS] = {{6, 48, 160, 0xFFFFFFFFu}, {8, 64, 0xFFFFFFFFu, 0xFFFFFFFFu}};
-    for (int k = 0; k < PACK_TIERS; ++k) { p.warps[k] = w[many][k]; p.evals[k] = e[many][k]; }
+    for (int k = 0; k < PACK_TIERS; ++k) { p.warps[k] = w[many][k]; p.evals[k] = e[many][k]; p.limit[k] = 0xFFFFFFFFu; }
+    // The last tiers answer a fault quickly, but only a few at a time on an SM. When the queue is some
+    // rounds long, a warp per fault on every slot of the heavy kernel gets through it sooner:
+    // the third tier hands its queue on, and the last leaves its own to the heavy kernel until
+    // few are left. (8,000 faults, nearly all heavy, of a chain of 1,000 levels, of 100 levels of 4
+    // nodes, of 50 levels of 64: 562, 48, 88 ms without these lines, 77, 11, 15 with, 80, 10, 15 with
+    // the light and heavy kernels. 60k nodes, 100k faults: 66 ms without, 84 with 32 and 2 per
+    // SM, 62 with 64 and 4. 500 faults of the chain: 92 ms with 64 and 4, 71 with 32 and 2.)
+    p.limit[2] = (uint32_t)((narrow ? 32u : 64u) * sms);
+    p.limit[3] = (uint32_t)((narrow ? 2u : 4u) * sms);
     p.use = true;
     return p;
 }
@@ -1603,16 +1627,19 @@ static int run_campaign(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_res
         CU(ctx->pk_prom_v.reserve(ctx->pk_prom_cap));
         CU(ctx->pk_cls.reserve(Fn));
     }
-    // behind the packed kernel the heavy kernel only takes the few faults no tier can hold
-    // for the rest of a window: cones of thousands of nodes, so 128 threads a fault unless the
-    // caller says (no-drop case of 10k nodes: 165 against 185 ms with one warp; designs whose node
-    // bitmap crowds shared memory keep the one-warp forms)
+    // Behind the packed tiers the heavy kernel takes the faults that no tier can hold for the rest of
+    // a window: few, with cones of thousands of nodes, so 128 threads each unless the caller says (no-drop
+    // case of 10k nodes: 165 against 185 ms with one warp; designs whose node bitmap crowds shared memory
+    // keep the one-warp forms). A second launch takes the last tier's crowds, a warp and a slot per
+    // fault, as in a run without the packed form.
+    const int cblock = pk.use && F > pk.limit[PACK_TIERS - 1] ? hblock : 0;   // 0: no crowd can gather
     if (pk.use && o.heavy_block <= 0) {
         uint32_t mnode = 0;
         for (Design *D : ctx->designs) mnode = std::max(mnode, D->N);
         if (mnode <= 400000) hblock = 128;
     }
-    rc = ensure_heavy_scratch(ctx, hblock, o.heavy_ctas > 0 || !pk.use ? o.heavy_ctas : 2 * ctx->n_sm, o.heavy_form);
+    rc = ensure_heavy_scratch(ctx, ctx->heavy, hblock, o.heavy_ctas > 0 || !pk.use ? o.heavy_ctas : 2 * ctx->n_sm, o.heavy_form);
+    if (rc == RTLFS_OK && cblock) rc = ensure_heavy_scratch(ctx, ctx->crowd, cblock, o.heavy_ctas, o.heavy_form);
     if (rc != RTLFS_OK) return rc;
     uint32_t *cinit = reinterpret_cast<uint32_t *>(ctx->p_small + 10);
     cinit[0] = n_heavy; cinit[1] = 0; cinit[2] = 0; cinit[3] = 0;
@@ -1643,9 +1670,9 @@ static int run_campaign(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_res
     if (per_sm < 1) return fail(ctx, RTLFS_E_ARG, "light kernel cannot be resident");
     const int lgrid = (int)std::max<int64_t>(1, std::min<int64_t>((ql.n_light + lblock - 1) / lblock,
                                                                    (int64_t)per_sm * ctx->n_sm));
-    const int hgrid = (int)ctx->heavy_grid;
+    const int hgrid = (int)ctx->heavy.grid;
     const int64_t lgrid_cap = (int64_t)per_sm * ctx->n_sm;
-    HeavyScratch hs = heavy_view(ctx);
+    const HeavyScratch hs = ctx->heavy.view(), hs_crowd = ctx->crowd.view();
     cudaEvent_t *ev = ctx->ev;
     uint32_t launches = 0;
 
@@ -1682,8 +1709,8 @@ static int run_campaign(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_res
         n32 = (3 + 2 * (PACK_TIERS - 1)) * (size_t)nw + 4 + PACK_TIERS;
         CU(ctx->w_cnt32.reserve(n32));
         // pool_top, light head, heavy head | packed (pk64): pool_top and head from the third tier to
-        // the heavy kernel | promotion pool top
-        n64 = (3 + 2 * (PACK_TIERS - 1)) * (size_t)nw + 2;
+        // the heavy kernel | promotion pool top | head of the crowds' launch
+        n64 = (4 + 2 * (PACK_TIERS - 1)) * (size_t)nw + 2;
         CU(ctx->w_cnt64.reserve(n64));
         while (ctx->ev_win.size() < 2 * WIN_TIMED * nw) {
             cudaEvent_t e;
@@ -1863,6 +1890,7 @@ static int run_campaign(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_res
             wl.fault_budget = o.fault_budget;
             wl.counters = ctx->d_heads.p + 4;
             if (!pk.use) CU(rec_time(ctx->ev_win[0 * nw + w], ctx->s_main));
+            PackArgs last{};   // the last tier's
             if (pk.use) {
                 // first tier on s_main, second on s_heavy, the others on s_tier (the heavy kernel
                 // behind the last): each takes what the tier before handed on in this window
@@ -1875,6 +1903,7 @@ static int run_campaign(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_res
                 for (int tier = 0; tier < PACK_TIERS && F; ++tier) {
                     PackArgs p = pa;
                     p.tier_evals = pk.evals[tier];
+                    p.tier_limit = pk.limit[tier];
                     p.items_out = ctx->pk_items[tier].p;
                     p.n_items_out = pk32 + 2 * PT * nw + tier;
                     if (tier == PACK_TIERS - 1) {   // emptied every window: its faults come back
@@ -1908,6 +1937,7 @@ static int run_campaign(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_res
                         p.item_begin = w == 0 ? zero : end + (w - 1);
                         p.item_end = end + w;
                         CU(cudaStreamWaitEvent(st, ctx->ev_pk[tier - 1], 0));
+                        last = p;
                     }
                     CU(rec_time(ctx->ev_win[2 * tier * (size_t)nw + w], st));
                     CU(launch_pack(tier, pk.multi, ctx->d_designs.p, pack_d0, f, p, pk.warps[tier], pk.grid, st));
@@ -1957,6 +1987,9 @@ static int run_campaign(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_res
                 wh.carry_out = ctx->pk_carry[k - 1][out].p;
                 wh.pool_r_out = ctx->pk_pool_r[k - 1][out].p; wh.pool_v_out = ctx->pk_pool_v[k - 1][out].p;
                 wh.n_carry_in = zero;
+                wh.cls = last.cls; wh.cap_regs = last.cap_regs; wh.cap_evals = last.cap_evals;
+                wh.prom_total = prom_total;
+                wh.counters_light = ctx->d_heads.p + 4;
                 wh.n_carry_out = pk32 + (PT + k - 1) * nw + w;
                 wh.pool_top_out = pk64 + (k - 1) * nw + w;
                 wh.pitems = ctx->pk_items[PACK_TIERS - 1].p;
@@ -1969,6 +2002,16 @@ static int run_campaign(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_res
             CU(rec_time(ctx->ev_win[2 * tk * nw + w], s_hv));
             CU(launch_heavy_window(ctx->d_designs.p, f, wh, hs, hblock, hgrid, s_hv));
             ++launches;
+            if (cblock) {   // the last tier's faults when they are too many for it
+                wh.carry_in = last.carry_in; wh.n_carry_in = last.n_carry_in;
+                wh.pool_r_in = last.pool_r_in; wh.pool_v_in = last.pool_v_in;
+                wh.pitems = last.items; wh.prom_begin = last.item_begin; wh.prom_end = last.item_end;
+                wh.prom_r = last.prom_r_in; wh.prom_v = last.prom_v_in;
+                wh.more_than = last.tier_limit;
+                wh.head = pk64 + 2 * PT * nw + 1 + w;
+                CU(launch_heavy_window(ctx->d_designs.p, f, wh, hs_crowd, cblock, (int)ctx->crowd.grid, s_hv));
+                ++launches;
+            }
             CU(rec_time(ctx->ev_win[(2 * tk + 1) * nw + w], s_hv));
         }
         CU(cudaEventRecord(ev[2], ctx->s_main));
@@ -2061,11 +2104,11 @@ static int run_campaign(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_res
                                      (uint64_t)dev_sched, (uint64_t)use_mlp, o.fault_budget, W, WU,
                                      (uint64_t)nodrop, (uint64_t)good_first, (uint64_t)o.order_classes,
                                      (uint64_t)pk.use, (uint64_t)pk.grid};
-        const void *ptrs[] = {ctx->d_designs.p, ctx->d_list_smem.p, ctx->d_list_glob.p, ctx->d_order.p, ctx->d_err.p, ctx->h_gbm.p,
+        const void *ptrs[] = {ctx->d_designs.p, ctx->d_list_smem.p, ctx->d_list_glob.p, ctx->d_order.p, ctx->d_err.p,
                               ctx->d_init_items.p, ctx->d_prom_items.p, ctx->d_heads.p, ctx->d_counters.p,
                               ctx->d_load.p, ctx->d_cycle.p, ctx->d_port.p, ctx->d_det.p, ctx->d_site.p,
                               ctx->d_bit.p, ctx->d_val.p, ctx->d_fdesign.p, ctx->p_cycle, ctx->p_port,
-                              ctx->p_det, ctx->p_load, ctx->h_fval.p, ctx->h_stamp.p, ctx->h_regr.p, ctx->h_regv.p,
+                              ctx->p_det, ctx->p_load,
                               ctx->d_X.p, ctx->d_heur.p, ctx->d_pred.p, ctx->d_mm.p, ctx->d_hist.p,
                               ctx->d_wb.p, ctx->d_static_ptrs.p, ctx->w_st_nreg.p, ctx->w_st_r.p,
                               ctx->w_st_v.p, ctx->w_live0.p, ctx->w_live1.p, ctx->w_cnt32.p, ctx->w_cnt64.p,
@@ -2079,8 +2122,10 @@ static int run_campaign(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_res
                                    (uint64_t)(uintptr_t)ctx->pk_pool_v[k >> 1][k & 1].p});
         const GoodLaunch &g = ctx->gl;
         key.insert(key.end(), {g.n_smem, g.n_glob, g.max_net_s, g.max_reg_s, g.max_ch_s, g.max_ch_g,
-                               ctx->hs_net, ctx->hs_reg, ctx->hs_node, ctx->hs_lv, (uint64_t)ctx->heavy_exact, (uint64_t)ctx->heavy_gbm,
                                (uint64_t)ctx->good_staging});
+        ctx->heavy.add_key(key);
+        ctx->crowd.add_key(key);
+        key.push_back((uint64_t)cblock);
         for (int lc = 1; lc < 5; ++lc)
             key.insert(key.end(), {(uint64_t)g.n_cl[lc], (uint64_t)g.smem_cl[lc],
                                    (uint64_t)(uintptr_t)ctx->d_list_cl[lc].p});
@@ -2171,7 +2216,7 @@ static int run_campaign(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_res
         st.promoted = cnts[0] - st.heavy_initial;
     }
     st.n_launches = launches;
-    st.heavy_form = pk.use ? 4u : ctx->heavy_gbm ? 3u : ctx->heavy_exact ? 1u : 2u;
+    st.heavy_form = pk.use ? 4u : ctx->heavy.use_gbm ? 3u : ctx->heavy.exact ? 1u : 2u;
     st.light_evals = heads[4];
     st.light_fault_cycles = heads[5];
     st.heavy_evals = heads[6];

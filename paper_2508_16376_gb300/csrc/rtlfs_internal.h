@@ -255,6 +255,11 @@ struct WinHeavy {
     unsigned long long *budget_hit;
     uint64_t fault_budget;
     uint32_t budget_at_end;       // as in PackArgs
+    uint32_t more_than;           // nothing is done unless there are more faults than this
+    uint8_t *cls;                 // null: every fault counts as heavy; else as in PackArgs
+    uint32_t cap_regs, cap_evals;
+    uint32_t *prom_total;
+    unsigned long long *counters_light;
     unsigned long long *counters;
     uint32_t *err;                // bit 1: pool overflow
 };
@@ -303,6 +308,8 @@ struct PackArgs {
     uint64_t prom_cap;
     uint8_t *cls;                 // [F] 1: the fault counts as heavy
     uint32_t tier_evals;          // a fault with more evaluations in a cycle goes to the next tier
+    uint32_t tier_limit;          // more faults than this all go to the next tier at once (the last
+                                  // tier leaves them to the heavy kernel)
     uint32_t cap_regs, cap_evals; // a light fault beyond these in a cycle counts as heavy
     uint32_t *prom_total;         // light faults that became heavy
     unsigned long long *budget_hit;

@@ -697,6 +697,10 @@ struct HeavyVars {
     uint32_t nd;               // exact form: words of the net bitmap to clear
     uint32_t nfr;              // fan-out ranges appended this cycle
     uint32_t nl;               // dirty nodes gathered for the current level
+    // thread 0's: whether the fault still counts as light, else since which cycle not, and its
+    // evaluations as a light one
+    uint32_t light, t_heavy;
+    unsigned long long load_light;
 };
 
 // Views of the heavy kernels' dynamic shared memory (heavy_smem_bytes sizes the same layout).
@@ -765,7 +769,7 @@ __device__ __forceinline__ void heavy_zero(const HeavySmem &m, const HeavyScratc
         for (uint32_t i = tid; i < HEAVY_FILTER / 32; i += B) m.flt[i] = 0;
     }
     for (uint32_t i = tid; i < m.nlw; i += B) m.lvm[i] = 0;
-    if (tid == 0) { V.nfr = 0; V.nl = 0; V.load = 0; }
+    if (tid == 0) { V.nfr = 0; V.nl = 0; V.load = 0; V.light = 0; }
 }
 
 // Outcome of one heavy fault's run.
@@ -777,6 +781,9 @@ struct HeavyRun {
     int32_t det_cycle, det_port;
     uint32_t mism;     // no-drop mode: cycles of this run with a differing output
     bool budget_at_end;   // in: the budget holds after cycle tend - 1 too
+    // The fault counts as light (V.light) until a cycle has more register diffs or evaluations than
+    // these.
+    uint32_t cap_regs, cap_evals;
 };
 
 // Simulate fault fid from cycle r.t until it is detected, exceeds the load budget or
@@ -1058,6 +1065,10 @@ __device__ __forceinline__ void heavy_run_fault(const DevDesign &D, const DevFau
         }
         if (my_load) atomicAdd(&V.load, (unsigned long long)my_load);
         __syncthreads();
+        if (tid == 0 && V.light) {
+            if (V.nreg_new > r.cap_regs || V.load - V.load_light > r.cap_evals) { V.light = 0; V.t_heavy = t; }
+            else V.load_light = V.load;
+        }
         if (EXACT) {   // clear the net bitmap for the next cycle
             const uint32_t nd = V.nd;
             if (nd <= HEAVY_DLIST) {
@@ -1387,7 +1398,13 @@ __device__ __forceinline__ void heavy_run_fault_warp(const DevDesign &D, const D
             if (lane == 0) cnt[L] = 0;
             ++L;
         }
-        load += __reduce_add_sync(FULL, my_load);
+        my_load = __reduce_add_sync(FULL, my_load);
+        if (lane == 0 && V.light && (V.nreg_new > r.cap_regs || my_load > r.cap_evals)) {
+            V.light = 0;
+            V.t_heavy = t;
+            V.load_light = load;
+        }
+        load += my_load;
         const uint32_t minport = __reduce_min_sync(FULL, pmin);
         __syncwarp();
         for (uint32_t i = lane; i < nlw; i += 32) lvm[i] = 0;
@@ -1499,12 +1516,13 @@ heavy_window_kernel(const DevDesign *__restrict__ designs, DevFaults f, WinHeavy
     uint32_t *regR = S.reg_r + (size_t)slot * 2 * S.max_reg;
     uint64_t *regV = S.reg_v + (size_t)slot * 2 * S.max_reg;
     uint32_t stamp = EXACT ? 0u : S.stamp[slot];   // the same in every thread, advanced together
-    heavy_zero<EXACT, GBM>(sm, S, V);
-    hsync<WARP>();
-
     // written before this launch by earlier work on the stream: the same in every thread
     const uint32_t n_carry = *q.n_carry_in, pb = *q.prom_begin, pe = *q.prom_end;
     const unsigned long long n_items = (unsigned long long)n_carry + (pe - pb);
+    if (n_items <= q.more_than) return;
+    heavy_zero<EXACT, GBM>(sm, S, V);
+    hsync<WARP>();
+
     for (;;) {
         if (tid == 0) s_item = atomicAdd(q.head, 1ull);
         hsync<WARP>();
@@ -1526,9 +1544,12 @@ heavy_window_kernel(const DevDesign *__restrict__ designs, DevFaults f, WinHeavy
             regR[k] = carried ? q.pool_r_in[cin.off + k] : q.pitems ? q.prom_r[pi.off + k] : it.reg_r[k];
             regV[k] = carried ? q.pool_v_in[cin.off + k] : q.pitems ? q.prom_v[pi.off + k] : it.reg_v[k];
         }
-        if (tid == 0) V.load = 0;
+        if (tid == 0) {
+            V.load = V.load_light = 0;
+            V.light = q.cls && !q.cls[fid];
+        }
         hsync<WARP>();
-        HeavyRun r{t_start, nreg0, 0, 0, -1, -1, 0, q.budget_at_end && tend < D.T};
+        HeavyRun r{t_start, nreg0, 0, 0, -1, -1, 0, q.budget_at_end && tend < D.T, q.cap_regs, q.cap_evals};
         if (WARP) heavy_run_fault_warp<EXACT, GBM>(D, f, fid, tend, q.fault_budget, sm, V, fval, stamp, regR, regV, S.max_reg, S.max_net, r);
         else heavy_run_fault<EXACT>(D, f, fid, tend, q.fault_budget, sm, V, fval, stamp, regR, regV, S.max_reg, S.max_net, r);
         hsync<WARP>();
@@ -1558,9 +1579,21 @@ heavy_window_kernel(const DevDesign *__restrict__ designs, DevFaults f, WinHeavy
                 f.res_port[fid] = r.det_port;
             }
             if (r.status == 3) atomicAdd(q.budget_hit, 1ull);
-            atomicAdd(q.counters + 0, V.load);
             const uint32_t t_end = r.status == 1 ? r.t + 1 : min(r.t, tend);
-            atomicAdd(q.counters + 1, (unsigned long long)(t_end - t_start));
+            uint32_t th = t_start;             // first cycle that counts as heavy,
+            unsigned long long l_light = 0;    // and the evaluations before it
+            if (q.cls && !q.cls[fid]) {
+                th = V.light ? t_end : V.t_heavy;
+                l_light = V.light ? V.load : V.load_light;
+                atomicAdd(q.counters_light + 0, l_light);
+                atomicAdd(q.counters_light + 1, (unsigned long long)(th - t_start));
+                if (!V.light) {
+                    q.cls[fid] = 1;
+                    atomicAdd(q.prom_total, 1u);
+                }
+            }
+            atomicAdd(q.counters + 0, V.load - l_light);
+            atomicAdd(q.counters + 1, (unsigned long long)(t_end - th));
         }
         hsync<WARP>();
     }

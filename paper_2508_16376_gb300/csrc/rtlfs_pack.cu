@@ -117,6 +117,8 @@ pack_kernel(const DevDesign *__restrict__ designs, const __grid_constant__ DevDe
     const uint32_t item0 = q.item_begin ? *q.item_begin : 0u;
     const uint32_t n_list = q.live_in ? (q.n_live_in ? *q.n_live_in : q.n_live) : *q.item_end - item0;
     const uint32_t n_items = n_carry + n_list;
+    const bool crowded = LPS > 1 && n_items > q.tier_limit;
+    if (BLOCK && crowded) return;   // the heavy kernel takes them
     // few faults: spread them over all units
     const uint32_t n_units = BLOCK ? gridDim.x : gridDim.x * (blockDim.x >> 5);
     const bool use_slot = slot < (n_items + n_units - 1) / n_units;
@@ -477,7 +479,7 @@ pack_kernel(const DevDesign *__restrict__ designs, const __grid_constant__ DevDe
                     ev_light = ev_heavy = 0;
                     mism = 0;
                     seen = nodrop && f.res_det[fid] == 1;
-                    if (nreg > R) {   // never fits this tier
+                    if (nreg > R || (LPS > 1 && crowded)) {   // never fits this tier, or too many do
                         next = PROMOTE;
                         continue;
                     }
