@@ -1085,26 +1085,33 @@ struct PackPlan {
 };
 
 // The packed form runs whenever its tags can name the levels of every design and 27 bits its
-// nets. A run that names a heavy form asks for the light and heavy kernels.
+// nets. A run that names a heavy form asks for the light and heavy kernels, and designs of registers
+// alone, where a cycle has nothing but its latches, are left to them (chains of 50 and 1,000 registers,
+// 800 and 2,000 faults over 600 cycles: 0.73 and 10.7 ms packed, 0.55 and 5.1 so).
 PackPlan plan_pack(rtlfs_ctx *ctx, int heavy_form) {
     PackPlan p;
-    uint32_t nl = 1, mn = 1;
+    uint32_t nl = 0, mn = 1;
     for (Design *D : ctx->designs) { nl = std::max(nl, D->n_levels); mn = std::max(mn, D->n_net); }
-    if (heavy_form != 0 || nl > PACK_LEVELS || mn > PACK_NETS) return p;
+    if (heavy_form != 0 || nl == 0 || nl > PACK_LEVELS || mn > PACK_NETS) return p;
     p.multi = ctx->designs.size() > 1;
     p.grid = ctx->n_sm;
     // With few faults the rounds of the slowest ones set the pace: faults move to a tier with
     // more lanes early. With many the issue slots do: they move only when their cones outgrow
     // what a tier handles in a few rounds, and the tiers' shares of an SM follow their work.
     // (medium campaign, 658 faults per SM, windows of 128: 922 against 1402 ms; transient list,
-    // 197 per SM, windows of 256: 199 against 182)
+    // 197 per SM, windows of 256: 199 against 182.) With thousands per SM nearly all the work is
+    // the first two tiers', and they get the warps: 1M faults of 1k, 3k, 10k, 30k nodes over 300
+    // cycles 85, 163, 238, 293 -> 53, 114, 182, 245 ms (light and heavy kernels: 76, 140, 240, 333).
+    // With 658 per SM over 10k cycles that costs a third; where levels are narrow it pays from
+    // some 1,500 (1k nodes, 300k faults: 29 -> 19 ms).
     bool narrow = true;   // levels narrower than four warps: a CTA has little over a warp
     for (Design *D : ctx->designs) narrow = narrow && D->N <= 128ull * D->n_levels;
     const uint64_t sms = (uint64_t)ctx->n_sm;
     const bool many = ctx->F > 400u * sms;
-    const int w[2][PACK_TIERS] = {{5, 4, 4, 1}, {3, 5, 7, 1}};
+    const int plan = ctx->F > (narrow ? 1500u : 4000u) * sms ? 2 : many;
+    const int w[3][PACK_TIERS] = {{5, 4, 4, 1}, {3, 5, 7, 1}, {8, 8, 3, 1}};
     const uint32_t e[2][PACK_TIERS] = {{6, 48, 160, 0xFFFFFFFFu}, {8, 64, 0xFFFFFFFFu, 0xFFFFFFFFu}};
-    for (int k = 0; k < PACK_TIERS; ++k) { p.warps[k] = w[many][k]; p.evals[k] = e[many][k]; p.limit[k] = 0xFFFFFFFFu; }
+    for (int k = 0; k < PACK_TIERS; ++k) { p.warps[k] = w[plan][k]; p.evals[k] = e[many][k]; p.limit[k] = 0xFFFFFFFFu; }
     // The last tiers answer a fault quickly, but only a few at a time on an SM. When the queue is some
     // rounds long, a warp per fault on every slot of the heavy kernel gets through it sooner:
     // the third tier hands its queue on, and the last leaves its own to the heavy kernel until
