@@ -521,6 +521,7 @@ int build_design(rtlfs_ctx *ctx, Design &D, const rtlfs_node *nodes, uint32_t N,
         r[2] = make_uint4(c[0], c[1], c[2], c[3]);
         r[3] = make_uint4(c[4], c[5], c[6], c[7]);
         r[4] = make_uint4(l[0] | l[1] << 16, l[2] | l[3] << 16, l[4] | l[5] << 16, l[6] | l[7] << 16);
+        if (e >= IR) r[5].x = D.lvl_start[D.node_level[e - IR] + 1];
     }
     D.chunks.clear();
     for (uint32_t l = 0; l < NL; ++l) {
@@ -2548,7 +2549,7 @@ int rtlfs_fault_sim_static(rtlfs_ctx *ctx, uint32_t design_id, const rtlfs_fault
         const size_t slots = std::min<size_t>((STATIC_SCRATCH_BYTES - L.thread_off) / L.per_thread, n_faults);
         const uint32_t per = (uint32_t)std::min<size_t>(warps, slots);
         const uint32_t blocks = (uint32_t)std::min<size_t>(slots / per, (size_t)16 * ctx->n_sm);
-        CU(launch_static(ctx->d_designs.p, design_id, D.N, D.n_net, faults, results, n_faults, blocks, per, arena, L, s));
+        CU(launch_static(ctx->d_designs.p, design_id, D.N, D.n_levels, D.n_net, faults, results, n_faults, blocks, per, arena, L, s));
     }
     for (uint32_t first = 0; warps == 0 && first < n_faults; first += wave) {
         const uint32_t cnt = std::min(wave, n_faults - first);

@@ -62,7 +62,8 @@ struct DevDesign {
     const uint4    *rec;        // [n_net][8] {nets of value slot 0, slot 1, select, meta (CONST: as desc)
                                 // | the slots the op reads << 4 | PM_*}, netinfo (z: the dreg_rec itself
                                 // when it is the only one), the first eight edges (2 x uint4), their
-                                // levels << 4 (8 x u16), unused: one 128-byte line per net
+                                // levels << 4 (8 x u16), {end of the node's level, unused}: one
+                                // 128-byte line per net
     const uint32_t *dreg_off;   // [n_net + 1] registers latching each net
     const uint32_t *dreg_idx;   // [n_dreg]
     const uint32_t *dreg_rec;   // [n_dreg] register index | register width << 25

@@ -83,6 +83,10 @@ __host__ __device__ inline size_t static_warp_bytes(uint32_t n_node, uint32_t n_
 // good one. What bounds it is the chain of a level, some 1000 cycles: the search for its nodes,
 // their 128-byte records, their operands. 1500 faults of 1200 nodes over 300 cycles: 13.0 ms with a
 // thread per fault and its heap of dirty nodes in the scratch array, 4.0 so.
+// THIN: for designs with a few nodes per level, where a level's search is most of its cost. 20 and
+// 2000 faults of a 1000-level chain over 50 cycles took 56 and 64 ms without the walk (a thread per
+// fault: 44 and 49), 18 and 22 with it. Elsewhere it costs 3% (1200 nodes), so it is left out there.
+template <bool THIN>
 __global__ void __launch_bounds__(128)
 static_kernel(const DevDesign *__restrict__ designs, uint32_t design, const StaticFault *__restrict__ faults,
               StaticResult *results, uint32_t n_faults, unsigned char *arena, StaticLayout L) {
@@ -144,12 +148,8 @@ static_kernel(const DevDesign *__restrict__ designs, uint32_t design, const Stat
                 atomicOr(m.bm + w, 1u << (n & 31u));
                 atomicOr(m.top + (w >> 5), 1u << (w & 31u));
             };
-            // a net that differs: its value, port, latches and consumers (ni: its netinfo)
-            auto keep = [&](uint32_t net, uint64_t v, uint64_t g, uint4 ni, const uint4 *r) {
-                val[net] = v;
-                const uint32_t w = net >> 5;
-                atomicOr(m.df + w, 1u << (net & 31u));
-                atomicOr(m.dtop + (w >> 5), 1u << (w & 31u));
+            // where a net that differs is seen: its port and latches (ni: its netinfo)
+            auto observe = [&](uint32_t net, uint64_t v, uint64_t g, uint4 ni) {
                 port = min(port, ni_port(ni.w));
                 uint32_t nl = ni_nreg(ni.w);
                 if (nl == 255u) nl = D.dreg_off[net + 1] - ni.z;
@@ -161,6 +161,14 @@ static_kernel(const DevDesign *__restrict__ designs, uint32_t design, const Stat
                     regr[nb * L.sreg + k] = rr & 0x1FFFFFFu;
                     regv[nb * L.sreg + k] = v & wm;
                 }
+            };
+            // and its value and consumers
+            auto keep = [&](uint32_t net, uint64_t v, uint64_t g, uint4 ni, const uint4 *r) {
+                observe(net, v, g, ni);
+                val[net] = v;
+                const uint32_t w = net >> 5;
+                atomicOr(m.df + w, 1u << (net & 31u));
+                atomicOr(m.dtop + (w >> 5), 1u << (w & 31u));
                 const uint32_t nf = ni.y - ni.x;
                 if (nf <= 8) {
                     const uint4 e0 = r[2], e1 = r[3];
@@ -201,12 +209,58 @@ static_kernel(const DevDesign *__restrict__ designs, uint32_t design, const Stat
                     break;
                 }
                 if (word == FULL) break;
-                // its level's dirty nodes in 32 words into the list: each lane reads and clears a word
-                // of its own, and the first lane's, which names the level, comes by a shuffle
+                // Each lane reads and clears a word of its own of the 32 looked at; the first one's
+                // lowest node n0 names the level.
                 const uint32_t wi = word + lane;
                 const uint32_t all = wi < nw ? m.bm[wi] : 0u;
-                const uint32_t n0 = word * 32 + __ffs((int)__shfl_sync(FULL, all, 0)) - 1;
-                const uint32_t end = __ldg(D.lvl_start + D.node_level[n0] + 1);
+                const uint32_t w0 = __shfl_sync(FULL, all, 0), n0 = word * 32 + __ffs((int)w0) - 1;
+                const uint4 *const r0 = rec + 8 * (size_t)(IR + n0);
+                const uint32_t end = __ldg(&r0[5].x);
+                auto operand = [&](uint4 d, uint32_t x, uint32_t bit) -> uint64_t {
+                    if (!(d.w & bit)) return 0ull;
+                    return m.df[x >> 5] >> (x & 31u) & 1u ? val[x] : __ldg(gcol + (size_t)x * T + t);
+                };
+                if constexpr (THIN) {
+                    // Alone in its level: the next dirty node n1 is one of a later level, or none of these
+                    // words. One lane walks on while what differs has a single consumer before n1: its value
+                    // stays in a register, and the consumer's record is on its way while the node's
+                    // operands are.
+                    const uint32_t rest = lane == 0 ? all & (all - 1) : all, more = __ballot_sync(FULL, rest != 0u);
+                    const uint32_t src = more ? __ffs((int)more) - 1 : 0u;
+                    const uint32_t wr = __shfl_sync(FULL, rest, src);
+                    const uint32_t n1 = more ? (word + src) * 32 + __ffs((int)wr) - 1 : (word + 32) * 32;
+                    if (n1 >= end) {
+                        if (lane == 0) {
+                            m.bm[word] = w0 & (w0 - 1);
+                            if (m.bm[word] == 0u) atomicAnd(m.top + (word >> 5), ~(1u << (word & 31u)));
+                            uint4 d = __ldg(r0), ni = __ldg(r0 + 1), e = __ldg(r0 + 2);
+                            uint64_t g = __ldg(gcol + (size_t)(IR + n0) * T + t);
+                            uint32_t net = IR + n0, fed = 0;   // fed: the slots that `fv` feeds, from bit 27
+                            uint64_t fv = 0;
+                            for (;;) {
+                                const uint32_t nx = e.x & (PACK_NETS - 1);
+                                const bool on = ni.y - ni.x == 1 && nx < IR + n1;
+                                const size_t to = on ? nx : net;   // no condition on the loads: their values are not merged
+                                const uint4 d2 = __ldg(rec + 8 * to), ni2 = __ldg(rec + 8 * to + 1), e2 = __ldg(rec + 8 * to + 2);
+                                const uint64_t g2 = __ldg(gcol + to * T + t);
+                                const uint64_t x = fed >> 27 & 1u ? fv : operand(d, d.x, 1u << 4), y = fed >> 28 & 1u ? fv : operand(d, d.y, 1u << 5);
+                                const uint64_t s = fed >> 29 & 1u ? fv : operand(d, d.z, 1u << 6);
+                                uint64_t v = pack_eval(d, x, y, s);
+                                if (net == site) v = force(v);
+                                if (v == g) break;
+                                if (!on) { keep(net, v, g, ni, rec + 8 * (size_t)net); break; }
+                                observe(net, v, g, ni);
+                                fed = e.x;
+                                fv = v;
+                                net = nx;
+                                d = d2; ni = ni2; e = e2; g = g2;
+                            }
+                        }
+                        __syncwarp();
+                        continue;
+                    }
+                }
+                // its dirty nodes into the list
                 uint32_t bits = 0, at = 0;
                 if (wi < nw && wi * 32 < end) {
                     bits = end - wi * 32 >= 32 ? all : all & ((1u << (end - wi * 32)) - 1u);
@@ -231,11 +285,7 @@ static_kernel(const DevDesign *__restrict__ designs, uint32_t design, const Stat
                     const uint4 *const r = rec + 8 * (size_t)net;
                     const uint4 d = __ldg(r), ni = __ldg(r + 1);
                     const uint64_t g = __ldg(gcol + (size_t)net * T + t);
-                    auto operand = [&](uint32_t x, uint32_t bit) -> uint64_t {
-                        if (!(d.w & bit)) return 0ull;
-                        return m.df[x >> 5] >> (x & 31u) & 1u ? val[x] : __ldg(gcol + (size_t)x * T + t);
-                    };
-                    const uint64_t x = operand(d.x, 1u << 4), y = operand(d.y, 1u << 5), s = operand(d.z, 1u << 6);
+                    const uint64_t x = operand(d, d.x, 1u << 4), y = operand(d, d.y, 1u << 5), s = operand(d, d.z, 1u << 6);
                     uint64_t v = pack_eval(d, x, y, s);
                     if (net == site) v = force(v);
                     if (v != g) keep(net, v, g, ni, r);
@@ -269,12 +319,14 @@ int static_warps(uint32_t n_node, uint32_t n_net) {
     return (int)std::min<size_t>(4, STATIC_SMEM / one);
 }
 
-cudaError_t launch_static(const DevDesign *d_designs, uint32_t design, uint32_t n_node, uint32_t n_net, const void *faults,
+cudaError_t launch_static(const DevDesign *d_designs, uint32_t design, uint32_t n_node, uint32_t n_levels, uint32_t n_net, const void *faults,
                           void *results, uint32_t n_faults, uint32_t blocks, uint32_t warps, void *arena, StaticLayout L, cudaStream_t stream) {
     const size_t smem = warps * static_warp_bytes(n_node, n_net);
-    cudaError_t e = cudaFuncSetAttribute(static_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // chains: where levels have a few nodes, one lane walks along them
+    const auto fn = n_node <= 8ull * n_levels ? static_kernel<true> : static_kernel<false>;
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    static_kernel<<<blocks, warps * 32, smem, stream>>>(d_designs, design, (const StaticFault *)faults, (StaticResult *)results,
+    fn<<<blocks, warps * 32, smem, stream>>>(d_designs, design, (const StaticFault *)faults, (StaticResult *)results,
                                                         n_faults, (unsigned char *)arena, L);
     return cudaGetLastError();
 }

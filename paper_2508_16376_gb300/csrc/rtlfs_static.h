@@ -32,7 +32,7 @@ cudaError_t static_scratch_address(int device, void **out);
 int static_warps(uint32_t n_node, uint32_t n_net);
 // `blocks` CTAs of `warps` (at most static_warps()) warps, a part of the scratch each (val u64 [net], register diffs
 // 2 x (u64 [sreg]), 2 x (u32 [sreg])); the word behind the error word counts faults from zero.
-cudaError_t launch_static(const DevDesign *d_designs, uint32_t design, uint32_t n_node, uint32_t n_net, const void *faults,
+cudaError_t launch_static(const DevDesign *d_designs, uint32_t design, uint32_t n_node, uint32_t n_levels, uint32_t n_net, const void *faults,
                           void *results, uint32_t n_faults, uint32_t blocks, uint32_t warps, void *arena, StaticLayout L, cudaStream_t stream);
 cudaError_t launch_plain_static(const DevDesign *d_designs, uint32_t design, const void *faults,
                                 void *results, uint32_t first, uint32_t count, void *arena,
