@@ -2424,6 +2424,8 @@ int rtlfs_mlp_set_weights(rtlfs_ctx *ctx, const uint16_t *w) {
     CU(cudaMemset(ctx->d_m.p, 0, MLP_PARAMS * sizeof(float)));
     CU(cudaMemset(ctx->d_v.p, 0, MLP_PARAMS * sizeof(float)));
     CU(cudaMemset(ctx->d_grad.p, 0, MLP_PARAMS * sizeof(float)));
+    rc = uploads_landed(ctx);
+    if (rc != RTLFS_OK) return rc;
     ctx->adam_step = 0;
     ctx->has_weights = true;
     return RTLFS_OK;
@@ -2438,14 +2440,15 @@ int rtlfs_mlp_get_weights(rtlfs_ctx *ctx, uint16_t *w) {
     return RTLFS_OK;
 }
 
+// On the stream of the kernels that read them: every caller waits for it before it returns.
 static int upload_samples(rtlfs_ctx *ctx, const float *X, const float *t, uint32_t n) {
     CU(ctx->d_tx.reserve((size_t)n * MLP_IN));
-    CU(cudaMemcpy(ctx->d_tx.p, X, (size_t)n * MLP_IN * sizeof(float), cudaMemcpyHostToDevice));
+    CU(cudaMemcpyAsync(ctx->d_tx.p, X, (size_t)n * MLP_IN * sizeof(float), cudaMemcpyHostToDevice, ctx->s_main));
     if (t) {
         CU(ctx->d_ty.reserve(n));
-        CU(cudaMemcpy(ctx->d_ty.p, t, (size_t)n * sizeof(float), cudaMemcpyHostToDevice));
+        CU(cudaMemcpyAsync(ctx->d_ty.p, t, (size_t)n * sizeof(float), cudaMemcpyHostToDevice, ctx->s_main));
     }
-    return uploads_landed(ctx);
+    return RTLFS_OK;
 }
 
 int rtlfs_mlp_forward(rtlfs_ctx *ctx, const float *X, uint32_t n, float *y) {
