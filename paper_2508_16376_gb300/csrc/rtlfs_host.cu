@@ -137,6 +137,10 @@ struct HeavySet {
         v.max_levels = max_levels;
         return v;
     }
+    void release() {
+        fval.release(); stamp.release(); regr.release(); regv.release(); gbm.release();
+        slots = grid = 0;
+    }
     // what a captured launch depends on
     void add_key(std::vector<uint64_t> &key) const {
         key.insert(key.end(), {(uint64_t)(uintptr_t)fval.p, (uint64_t)(uintptr_t)stamp.p, (uint64_t)(uintptr_t)regr.p,
@@ -1049,6 +1053,7 @@ int ensure_heavy_scratch(rtlfs_ctx *ctx, HeavySet &h, int block, int want_slots,
     const bool grow = slots > (int)h.slots || mn > h.max_net || mr > h.max_reg;
     if (grow) {
         h.fval.release(); h.regr.release(); h.regv.release(); h.stamp.release();
+        h.slots = 0;   // until all of it is there
         CU(h.fval.reserve((size_t)slots * mn));
         CU(h.stamp.reserve((size_t)slots));
         h.stamps_stale = true;   // fresh memory: zeroed below before a stamped run
@@ -1551,10 +1556,10 @@ static int run_good_only(rtlfs_ctx *ctx) {
 }
 
 // One campaign. packed_ok = false: the light and heavy kernels even where the packed form could
-// run. *overflow: the packed form ran out of room for register diffs.
+// run. *packed: the packed form was to run it; *overflow: it ran out of room for register diffs.
 static int run_campaign(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_result *const *out,
-                        uint64_t *const *out_load, bool packed_ok, bool *overflow) {
-    *overflow = false;
+                        uint64_t *const *out_load, bool packed_ok, bool *packed, bool *overflow) {
+    *packed = *overflow = false;
     if (!ctx) return RTLFS_E_ARG;
     if (ctx->designs.empty()) return fail(ctx, RTLFS_E_STATE, "no design loaded");
     if (!out) return fail(ctx, RTLFS_E_ARG, "null result array");
@@ -1593,6 +1598,7 @@ static int run_campaign(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_res
     // faults start as heavy ones, and does not wait for the 256 cycles of good trace that a
     // score needs (large design over 512 cycles: 72 against 91 ms).
     PackPlan pk = packed_ok ? plan_pack(ctx, o.heavy_form) : PackPlan{};
+    *packed = pk.use;
     const bool scored = o.scheduler == RTLFS_SCHED_HEURISTIC ? !pk.use || o.heavy_frac > 0.f : o.scheduler != RTLFS_SCHED_PLAIN;
     const bool dev_sched = scored && F > 0;
     const bool use_mlp = o.scheduler == RTLFS_SCHED_MLP && ctx->has_weights;
@@ -2255,11 +2261,32 @@ static int run_campaign(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_res
     return RTLFS_OK;
 }
 
+// What only the packed form holds, and the windowed form's buffers, which it also uses in one pass.
+static void release_packed(rtlfs_ctx *ctx) {
+    for (auto &b : ctx->pk_items) b.release();
+    ctx->pk_prom_r.release(); ctx->pk_prom_v.release(); ctx->pk_last_r.release(); ctx->pk_last_v.release();
+    ctx->pk_cls.release();
+    for (int k = 0; k < PACK_TIERS - 2; ++k)
+        for (int b = 0; b < 2; ++b) {
+            ctx->pk_carry[k][b].release(); ctx->pk_pool_r[k][b].release(); ctx->pk_pool_v[k][b].release();
+        }
+    ctx->w_st_nreg.release(); ctx->w_st_r.release(); ctx->w_st_v.release(); ctx->w_live0.release(); ctx->w_live1.release();
+    ctx->w_carry0.release(); ctx->w_carry1.release();
+    ctx->w_pool_r0.release(); ctx->w_pool_r1.release(); ctx->w_pool_v0.release(); ctx->w_pool_v1.release();
+    ctx->crowd.release();
+}
+
 int rtlfs_run(rtlfs_ctx *ctx, const rtlfs_run_opts *opts, rtlfs_result *const *out, uint64_t *const *out_load) {
-    bool overflow = false;
-    const int rc = run_campaign(ctx, opts, out, out_load, true, &overflow);
-    // more register diffs than the packed form's pools hold: the light and heavy kernels
-    return overflow ? run_campaign(ctx, opts, out, out_load, false, &overflow) : rc;
+    bool packed = false, overflow = false;
+    const int rc = run_campaign(ctx, opts, out, out_load, true, &packed, &overflow);
+    if (rc != RTLFS_E_NOMEM || !packed) return rc;
+    // More register diffs than the packed form's pools hold, or no room for them on the device:
+    // the light and heavy kernels, which need far less.
+    if (!overflow) {
+        cudaGetLastError();   // the failed allocation's, or the next launch reports it
+        release_packed(ctx);
+    }
+    return run_campaign(ctx, opts, out, out_load, false, &packed, &overflow);
 }
 
 int rtlfs_run_plain(rtlfs_ctx *ctx, rtlfs_result *const *out) {
