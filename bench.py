@@ -493,8 +493,9 @@ def main():
         shard.gather_results(my_results, mine, [len(f) for _, _, f in parts])
 
     last = stats[-1]
-    mean = {k: float(np.mean([s[k] for s in stats])) for k in ("good_ms", "light_ms", "heavy_ms")}
-    n_win = roofline.windows(run_opts, max(s.shape[0] for _, s, _ in my_parts))
+    mean = roofline.kernel_times(stats, dev_ms)
+    n_win = (int(last["n_launches"]) if "packed_ms" in mean
+             else roofline.windows(run_opts, max(s.shape[0] for _, s, _ in my_parts)))
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": ws, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms_all, "higher_is_better": True,
             "scaling": "strong", "vs_baseline": None, "dtype": "u64", "data": "synthetic",

@@ -10,8 +10,8 @@ HBM bytes per step:
 * the stimulus read once: 8 B x inputs x cycles;
 * the per-fault state carried across cycle-window boundaries: every fault still alive at a
   boundary writes and reads its live-list entry (4 B) and register-diff count (1 B), 10 B
-  per crossing (the register-diff entries themselves are not counted: the library's
-  counters do not record them);
+  per crossing of the caller's windows (the register-diff entries themselves are not counted:
+  the library's counters do not record them; nor are the packed form's shorter windows);
 * the fault descriptors read (8 B) and the results (cycle, port, detected: 9 B) and loads
   (8 B) written once per fault.
 
@@ -81,7 +81,8 @@ def heavy_traffic_per_launch(stats: dict, n_win: int, gbm_form: bool) -> Optiona
 
 
 def windows(run_opts: dict, T: int) -> int:
-    """Launches of each window kernel per campaign."""
+    """Launches of each window kernel per campaign (the light and heavy kernels': the packed form
+    chooses its own windows and launches several kernels in each)."""
     W = int(run_opts.get("window", 0) or 0)
     return -(-int(T) // W) if W else 1
 
@@ -136,11 +137,24 @@ def int_peak(peaks: dict, sm_mhz: Optional[float], n_sm: int = N_SM) -> dict:
             "lanes_per_sm": INT32_LANES_PER_SM, "sm_mhz": mhz}
 
 
+def kernel_times(stats: List[dict], step_ms: float) -> dict:
+    """Mean kernel times of the steps, for dominant(). The packed form's heavy_ms adds up tiers
+    that run side by side, so its kernels are taken together: the span of the faulty machines, or
+    under graph replay, which does not time it, the step."""
+    mean = {k: float(np.mean([s[k] for s in stats])) for k in ("good_ms", "light_ms", "heavy_ms")}
+    if stats[-1].get("heavy_form") == 4:
+        mean["packed_ms"] = float(np.mean([s["faulty_ms"] for s in stats])) or step_ms
+    return mean
+
+
 def dominant(mean_ms: dict):
-    """The faulty-machine kernel with the larger summed launch time. The good trace is not a
+    """The faulty-machine kernel with the larger summed launch time, or the packed form's kernels
+    together. The good trace is not a
     candidate: in the windowed campaign its figure is the span of its stream, which waits for
     SMs behind the persistent faulty kernels (its kernels' own share of a serialised launch
     list is a few percent)."""
+    if "packed_ms" in mean_ms:
+        return "packed", mean_ms["packed_ms"]
     name = max(("light_ms", "heavy_ms"), key=lambda k: mean_ms[k])
     return {"light_ms": "light", "heavy_ms": "heavy"}[name], mean_ms[name]
 
