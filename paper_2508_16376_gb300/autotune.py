@@ -10,8 +10,11 @@ kept in fault-list order).
 Every candidate is timed with real campaigns through rtlfs_run on the workload loaded in
 the simulator (device-event time of the whole campaign, best of `repeats`). The search is
 coordinate descent: starting from BASE, each knob in turn takes the value that times
-fastest with the others held at the best so far, for `passes` passes. Results never depend
-on the knobs, so tuning changes only time. Winners are cached per size bucket (log2 of
+fastest with the others held at the best so far, for `passes` passes. Where the library runs the
+packed form (BASE's runs say so), the knobs that only decide how its counters class a fault,
+or that it replaces with its own (BLIND), are left alone, and a second descent names the light
+and heavy kernels (heavy_form 1), whose knobs they are; the faster of the two forms wins. Results
+never depend on the knobs, so tuning changes only time. Winners are cached per size bucket (log2 of
 total nets, cycles and faults, and the design count) in a JSON file next to this module.
 """
 from __future__ import annotations
@@ -37,6 +40,9 @@ KNOBS: List[Tuple[str, Sequence]] = [
     ("good_first", (0, 1)),
     ("order_classes", (0, 8, 1)),
 ]
+
+PACKED_FORM = 4   # rtlfs_stats.heavy_form
+BLIND = ("window", "light_cap", "light_block")
 
 
 def fixed_opts(sim, with_mlp: bool) -> Dict:
@@ -99,15 +105,24 @@ def tune(sim, repeats: int = 1, passes: int = 1, cache_path: str = CACHE, use_ca
                 print(f"autotune {key}: {opts} -> {ms:.1f} ms", flush=True)
         return timed[k]
 
-    best = dict(BASE, **fixed)
-    best_ms = time_of(best)
-    for _ in range(passes):
-        for name, values in (knobs or KNOBS):
-            for v in values:
-                cand = dict(best, **{name: v})
-                ms = time_of(cand)
-                if ms < best_ms:
-                    best, best_ms = cand, ms
+    def descend(best: Dict, blind: Sequence[str] = ()) -> Tuple[float, Dict]:
+        best_ms = time_of(best)
+        for _ in range(passes):
+            for name, values in (knobs or KNOBS):
+                for v in values if name not in blind else ():
+                    cand = dict(best, **{name: v})
+                    ms = time_of(cand)
+                    if ms < best_ms:
+                        best, best_ms = cand, ms
+        return best_ms, best
+
+    base = dict(BASE, **fixed)
+    time_of(base)
+    if sim.stats().get("heavy_form") == PACKED_FORM:
+        packed = descend(base, BLIND)
+        best_ms, best = min(packed, descend(dict(base, heavy_form=1)), key=lambda x: x[0])
+    else:
+        best_ms, best = descend(base)
     if use_cache:
         cache = _load_cache(cache_path)
         cache[key] = dict(opts=best, ms=best_ms, trials=trials)
