@@ -2503,7 +2503,7 @@ int rtlfs_mlp_grad(rtlfs_ctx *ctx, const float *X, const float *t, uint32_t n, f
     if (rc != RTLFS_OK) return rc;
     CU(cudaMemsetAsync(ctx->d_grad.p, 0, MLP_PARAMS * sizeof(float), ctx->s_main));
     CU(cudaMemsetAsync(ctx->d_loss.p, 0, sizeof(float), ctx->s_main));
-    CU(launch_mlp_grad(ctx->d_wb.p, ctx->d_tx.p, ctx->d_ty.p, n, ctx->d_grad.p, ctx->d_loss.p, ctx->s_main));
+    CU(launch_mlp_grad(ctx->d_wb.p, ctx->d_tx.p, ctx->d_ty.p, n, ctx->d_grad.p, ctx->d_loss.p, (uint32_t)ctx->n_sm, ctx->s_main));
     float lsum = 0.f;
     CU(cudaMemcpyAsync(grad, ctx->d_grad.p, MLP_PARAMS * sizeof(float), cudaMemcpyDeviceToHost, ctx->s_main));
     CU(cudaMemcpyAsync(&lsum, ctx->d_loss.p, sizeof(float), cudaMemcpyDeviceToHost, ctx->s_main));
@@ -2527,7 +2527,7 @@ int rtlfs_mlp_train(rtlfs_ctx *ctx, const float *X, const float *t, uint32_t n, 
         for (uint32_t s0 = 0; s0 < n; s0 += batch) {
             const uint32_t nb = std::min(batch, n - s0);
             CU(launch_mlp_grad(ctx->d_wb.p, ctx->d_tx.p + (size_t)s0 * MLP_IN, ctx->d_ty.p + s0, nb,
-                               ctx->d_grad.p, ctx->d_loss.p, ctx->s_main));
+                               ctx->d_grad.p, ctx->d_loss.p, (uint32_t)ctx->n_sm, ctx->s_main));
             CU(launch_mlp_adam(ctx->d_master.p, ctx->d_wb.p, ctx->d_grad.p, ctx->d_m.p, ctx->d_v.p, lr,
                                0.9f, 0.999f, 1e-8f, ++ctx->adam_step, ctx->s_main));
         }

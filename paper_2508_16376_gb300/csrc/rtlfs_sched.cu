@@ -462,12 +462,12 @@ cudaError_t launch_mlp_forward(const void *wb, const float *X, uint32_t n, float
 }
 
 cudaError_t launch_mlp_grad(const void *wb, const float *X, const float *t, uint32_t n, float *grad,
-                            float *loss_sum, cudaStream_t s) {
+                            float *loss_sum, uint32_t n_sm, cudaStream_t s) {
     if (!n) return cudaSuccess;
-    // Tiles of 128 samples when they fill the 152 SMs, else of 32, for more CTAs; two CTAs per SM
+    // Tiles of 128 samples when they fill the SMs (152: from 19456 samples), else of 32, for more CTAs; two per SM
     // (65537 samples, the call: 123 us; one CTA per SM 127-135, tiles of 64 126).
-    const bool big = n >= 152u * 128u;
-    const uint32_t S = big ? 128 : 32, tiles = n / S + (n % S != 0), grid = tiles < 304u ? tiles : 304u;
+    const bool big = n >= n_sm * 128u;
+    const uint32_t S = big ? 128 : 32, tiles = n / S + (n % S != 0), grid = tiles < 2 * n_sm ? tiles : 2 * n_sm;
     const size_t smem = (big ? grad_floats<8>() : grad_floats<2>()) * sizeof(float);
     const auto fn = big ? mlp_grad_kernel<8> : mlp_grad_kernel<2>;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

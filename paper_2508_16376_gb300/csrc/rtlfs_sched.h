@@ -21,7 +21,7 @@ cudaError_t launch_features(const DevDesign *d_designs, DevFaults f, const float
                             float *X, float *heur, cudaStream_t s, uint32_t t_limit = TOGGLE_CYCLES);
 cudaError_t launch_mlp_forward(const void *wb, const float *X, uint32_t n, float *y, cudaStream_t s);
 cudaError_t launch_mlp_grad(const void *wb, const float *X, const float *t, uint32_t n, float *grad,
-                            float *loss_sum, cudaStream_t s);
+                            float *loss_sum, uint32_t n_sm, cudaStream_t s);
 cudaError_t launch_mlp_adam(float *master, void *wb, float *grad, float *m, float *v, float lr,
                             float beta1, float beta2, float eps, int step, cudaStream_t s);
 // Orders the n faults by descending score into order[]; the first n_heavy become heavy
