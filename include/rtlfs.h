@@ -142,9 +142,13 @@ typedef struct {
     float    heavy_frac;     /* fraction of faults (highest predicted load) sent to the
                                 heavy kernel from cycle 0; < 0 = auto */
     int32_t  use_graph;      /* 1 = capture the launch sequence in a CUDA graph and replay */
-    uint64_t fault_budget;   /* max node evaluations per fault, 0 = unlimited */
+    uint64_t fault_budget;   /* max node evaluations per fault, 0 = unlimited; looked at after
+                                every simulated cycle but the last of a `window` */
     int32_t  light_cap;      /* light-lane capacity variant: 1 = 4 register diffs / 12 net
-                                diffs / 12 pending nodes, 2 = 8/24/24, 3 = 8/48/48; 0 = auto */
+                                diffs / 12 pending nodes, 2 = 8/24/24, 3 = 8/48/48; 0 = auto.
+                                The packed form counts a fault as heavy from the first cycle
+                                with more register diffs, or more evaluations than the variant
+                                has pending nodes */
     int32_t  window;         /* cycles per window: every live fault advances through the same
                                 window of cycles, the good trace of the next window, the light
                                 kernel and the heavy kernel overlap on three streams; 0 = each
@@ -162,12 +166,21 @@ typedef struct {
                                 options must match the stopped run's window, no_drop and
                                 light_cap (RTLFS_E_ARG otherwise) */
     int32_t  heavy_form;     /* 0 = auto: the packed form (several faults per warp, in tiers of 1, 8,
-                                32 and 256 lanes per fault; windows of 64 cycles inside the ones
-                                asked for; light and heavy options then only decide which faults
-                                the counters call light or heavy) for designs of at most 4095
-                                levels and 2^27 nets, else as 1 unless its bitmap costs resident
-                                CTAs. Otherwise the light and heavy kernels with this record of
-                                differing nets: 1 = a shared-memory
+                                32 and 256 lanes per fault; the heavy kernel behind the last tier
+                                takes the faults that no tier holds, and all of the last tier's
+                                where they are too many for it; windows of 64 cycles inside the
+                                ones asked for; light_block, and the light and heavy options but
+                                heavy_block and heavy_ctas, then only decide which faults the
+                                counters call light or heavy) for designs with nodes, of at most
+                                4095 levels and 2^27 nets, else as 1 unless its bitmap costs
+                                resident CTAs. Beside the buffers of a windowed run it holds five
+                                more pools of register diffs (12 B each, faults x registers of
+                                them, at most 16 M) and one of faults handed on (12 B each, 164
+                                per fault, at most 64 M), some 1.8 GB at most; where an
+                                allocation fails, or a pool runs over, the campaign runs on the
+                                light and heavy kernels (for a pool that runs over, from its
+                                start: stats describe the second run). Otherwise the light and
+                                heavy kernels with this record of differing nets: 1 = a shared-memory
                                 bit per net, 2 = a small shared filter plus cycle stamps on
                                 the values in global scratch (for designs whose per-net
                                 bitmap would crowd shared memory), 3 = as 2 with the
@@ -209,7 +222,9 @@ typedef struct {
                                 each one's own time summed (they overlap) */
     uint64_t fault_cycles;   /* W = sum over faults of (cycle+1 if detected else T) */
     uint64_t node_evals;     /* sum of the per-fault propagation loads */
-    uint64_t promoted;       /* light faults promoted to the heavy kernel */
+    uint64_t promoted;       /* light faults promoted to the heavy kernel, or, in the packed form,
+                                that became heavy by light_cap's rule; the two rules differ, so do
+                                the counts (and the light and heavy ones below; sums agree) */
     uint64_t heavy_initial;  /* faults assigned to the heavy kernel from cycle 0 */
     uint32_t n_launches;     /* kernels launched by the run */
     uint32_t heavy_form;     /* heavy kernel's record of differing nets in the run: 1 exact,

@@ -373,8 +373,9 @@ int build_design(rtlfs_ctx *ctx, Design &D, const rtlfs_node *nodes, uint32_t N,
     if (N == 0) NL = 0;
     if (NL > 65535) return fail(ctx, RTLFS_E_ARG, "more than 65535 levels");
 
-    // Renumber: nodes sorted by (level, op, index). Grouping a level's nodes by op keeps
-    // the 32 nodes a warp evaluates together on one branch of the op switch.
+    // Renumber: nodes sorted by (level, op, index). Grouping a level's nodes by op keeps the nodes a warp
+    // evaluates together on one branch of the op switch where a kernel has one (the light and heavy
+    // kernels and the staged and global good traces; the others evaluate every op in one straight line).
     D.I = I; D.R = R; D.N = N; D.O = O; D.n_net = n_net; D.n_levels = NL;
     D.lvl_start.assign(NL + 1, 0);
     for (uint32_t n = 0; n < N; ++n) ++D.lvl_start[level[n] + 1];
@@ -1102,7 +1103,7 @@ PackPlan plan_pack(rtlfs_ctx *ctx, int heavy_form) {
     p.multi = ctx->designs.size() > 1;
     p.grid = ctx->n_sm;
     // With few faults the rounds of the slowest ones set the pace: faults move to a tier with
-    // more lanes early. With many the issue slots do: they move only when their cones outgrow
+    // more lanes early. With many the few warps that fit an SM do: they move only when their cones outgrow
     // what a tier handles in a few rounds, and the tiers' shares of an SM follow their work.
     // (medium campaign, 658 faults per SM, windows of 128: 922 against 1402 ms; transient list,
     // 197 per SM, windows of 256: 199 against 182.) With thousands per SM nearly all the work is

@@ -92,7 +92,7 @@ struct DevDesign {
 // four bytes select the terms of the bitwise result. A constant reads its own net, set up once.
 constexpr uint32_t GM_A = 1u << 7, GM_B = 1u << 15, GM_C = 1u << 23, GM_D = 1u << 31;
 constexpr uint32_t GM_LEFT = 1u << 16, GM_SUM = 1u << 17, GM_CMP = 1u << 18, GM_EQ = 1u << 19;
-constexpr uint32_t GM_NEG = 1u << 20, GM_MUX = 1u << 21, GM_LAST = 1u << 24, GM_VALID = 1u << 25;
+constexpr uint32_t GM_NEG = 1u << 20, GM_MUX = 1u << 21, GM_VALID = 1u << 25;
 
 // Evaluation masks of a packed record's meta (pack_eval).
 constexpr uint32_t PM_LEFT = 1u << 24, PM_SUM = 1u << 25, PM_CMP = 1u << 26;

@@ -22,22 +22,27 @@
 //
 // Tiers: one lane per fault for the many faults with a handful of dirty nodes, then 8, a warp,
 // and a CTA of 256. A fault that outgrows its table or buffer is handed to the next tier
-// with its start-of-cycle register diffs (behind the last is the heavy kernel, with its
-// state in global memory). Which faults count as light or heavy (evaluation counters,
-// promotions) follows the light lanes' capacity rule and does not depend on the tier.
+// with its start-of-cycle register diffs; behind the last is the heavy kernel, with its
+// state in global memory, which also takes the last tier's faults where they are too many for it
+// (plan_pack). Which faults count as light or heavy (evaluation counters, promotions) does not
+// depend on the tier or on the kernel: a fault is heavy from the first cycle with more
+// evaluations or register diffs than light_cap names. (The light kernel promotes by what is pending or
+// differs at once instead, so the two forms' counts differ; their sums do not.)
 //
-// What bounds it: instructions, not memory. A round is about 250 warp instructions at 7 cycles
-// each (ncu, medium campaign, 32 lanes per fault: 2.3 of them fixed latency, 1.5 L2 loads, 1.1
-// branches), so a fault's pace is its levels times about a microsecond, and the throughput is
-// the issue slots: 3.1e9 warp instructions per 128 cycles of the medium campaign against 6.4e9
-// of a lane and a warp per fault. Light and heavy kernels -> now (whole calls, with the good
-// trace's own gains): tiny list 6.8 -> 2.4 ms, 2.8k nodes 61 -> 15 ms, 20k nodes with 5k faults 286 -> 82
-// ms, with 100k faults over 10k cycles 1125 -> 881 ms, transient list 270 -> 152 ms, no-drop 131 -> 72 ms,
-// twelve designs 193 -> 89 ms, 200k nodes 169 -> 62 ms.
+// What bounds it: a warp instruction takes 7 to 8 cycles (2.2 of fixed latency, 1.2-1.9 of global
+// loads, 1.1 of branches), and a warp's tables take 9 to 15 KB of shared memory, so 3 to 7 warps a
+// tier are resident on an SM. With many faults (20k nodes, 100k faults, a window of 64 cycles) the
+// tiers issue in 12 to 22% of the slots, 16% for the busiest; with few (5,003 faults) a tier lasts as
+// long as its slowest fault's chain of rounds, about a microsecond per level. Neither memory nor
+// issue is near a limit. Light and heavy kernels -> packed (whole calls, with the good trace's own
+// gains): tiny list 6.8 -> 2.4 ms, 2.8k nodes 61 -> 15 ms, 20k nodes with 5k faults 286 -> 82 ms, with
+// 100k faults over 10k cycles 1125 -> 850 ms, transient list 270 -> 152 ms, no-drop 131 -> 72 to 80 ms, twelve
+// designs 193 -> 88 ms, 200k nodes 169 -> 62 to 65 ms.
 // With few faults the last tier sets the pace, and its level the barriers and instructions of its
-// rounds. Slower there: items listed and dealt to the lanes evenly (recorded loads 103 against 83
-// ms: few rounds have two items on a lane), consumers' records prefetched into L1 when they are
-// marked (88), 128 or 64 lanes (no-drop 247, 258 against 115: tables overflow).
+// rounds. Slower there (before its reductions took one barrier): items listed and dealt to the lanes
+// evenly (recorded loads 103 against 83 ms: few rounds have two items on a lane), consumers' records
+// prefetched into L1 when they are marked (88), 128 or 64 lanes (no-drop with another fault list 247,
+// 258 against 115: tables overflow).
 #include "rtlfs_device.h"
 #include "rtlfs_internal.h"
 
