@@ -1647,14 +1647,23 @@ static int run_campaign(rtlfs_ctx *ctx, const rtlfs_run_opts *opts_in, rtlfs_res
     // case of 10k nodes: 165 against 185 ms with one warp; designs whose node bitmap crowds shared memory
     // keep the one-warp forms). A second launch takes the last tier's crowds, a warp and a slot per
     // fault, as in a run without the packed form.
-    const int cblock = pk.use && F > pk.limit[PACK_TIERS - 1] ? hblock : 0;   // 0: no crowd can gather
+    int cblock = pk.use && F > pk.limit[PACK_TIERS - 1] ? hblock : 0;   // 0: no crowd can gather
     if (pk.use && o.heavy_block <= 0) {
         uint32_t mnode = 0;
         for (Design *D : ctx->designs) mnode = std::max(mnode, D->N);
         if (mnode <= 400000) hblock = 128;
     }
     rc = ensure_heavy_scratch(ctx, ctx->heavy, hblock, o.heavy_ctas > 0 || !pk.use ? o.heavy_ctas : 2 * ctx->n_sm, o.heavy_form);
-    if (rc == RTLFS_OK && cblock) rc = ensure_heavy_scratch(ctx, ctx->crowd, cblock, o.heavy_ctas, o.heavy_form);
+    if (rc == RTLFS_OK && cblock) {
+        rc = ensure_heavy_scratch(ctx, ctx->crowd, cblock, o.heavy_ctas, o.heavy_form);
+        if (rc == RTLFS_E_NOMEM) {   // its slots are most of what the light and heavy kernels need: the tiers take all
+            cudaGetLastError();
+            ctx->crowd.release();
+            cblock = 0;
+            for (uint32_t &l : pk.limit) l = 0xFFFFFFFFu;
+            rc = RTLFS_OK;
+        }
+    }
     if (rc != RTLFS_OK) return rc;
     uint32_t *cinit = reinterpret_cast<uint32_t *>(ctx->p_small + 10);
     cinit[0] = n_heavy; cinit[1] = 0; cinit[2] = 0; cinit[3] = 0;

@@ -34,3 +34,32 @@ def test_run_without_room_for_the_pools(opts):
         assert form in (1, 2, 3) and sim.stats()["heavy_form"] == 4
     for r, l in ((got, gl), (again, al)):
         assert np.array_equal(r[0], ref[0]) and np.array_equal(l[0], rl[0])
+
+
+def test_run_without_room_for_the_crowds():
+    """Room for the packed form but not for a slot per resident warp of the heavy kernel: the tiers take every fault."""
+    import torch
+    from paper_2508_16376_gb300 import build
+    build.build()
+    d = synth.gen_datapath_fsm(5, 60000, 64, 16, 16, [8], 0.8, 24, 64)
+    u = synth.fault_universe(d)
+    f = u.take(np.sort(np.random.default_rng(2).choice(len(u), 3000, replace=False)))
+    stim = synth.stimulus(d, 70, 3, 0.1)
+    with Simulator(0) as sim:
+        sim.add(d, stim, f)
+        ref, rl = sim.run(want_load=True, heavy_form=1)
+    with Simulator(0) as sim:
+        sim.add(d, stim, f)
+        free, _ = torch.cuda.mem_get_info()
+        hog = torch.empty(max(0, free - (1200 << 20)), dtype=torch.uint8, device="cuda")   # the slots take 3 GB
+        try:
+            got, gl = sim.run(want_load=True)
+            form = sim.stats()["heavy_form"]
+            again, al = sim.run(want_load=True, use_graph=1, window=64)
+        finally:
+            del hog
+            torch.cuda.empty_cache()
+        roomy, ml = sim.run(want_load=True, use_graph=1, window=64)
+        assert form == 4 and sim.stats()["heavy_form"] == 4
+    for r, l in ((got, gl), (again, al), (roomy, ml)):
+        assert np.array_equal(r[0], ref[0]) and np.array_equal(l[0], rl[0])
