@@ -321,6 +321,8 @@ struct PackArgs {
 };
 
 size_t pack_smem_bytes(int tier, int warps);
+// The records of a design (DevDesign::rec) from its other arrays.
+cudaError_t launch_records(const DevDesign &d, uint4 *rec, cudaStream_t stream);
 // d0: the design when there is only one (multi = false).
 cudaError_t launch_pack(int tier, bool multi, const DevDesign *d_designs, const DevDesign &d0, DevFaults f,
                         const PackArgs &q, int warps, int grid, cudaStream_t stream);

@@ -660,6 +660,59 @@ pack_kernel(const DevDesign *__restrict__ designs, const __grid_constant__ DevDe
     if (acc3) atomicAdd(q.counters_heavy + 1, acc3);
 }
 
+// Everything the packed kernel reads of a net in one 128-byte record, a thread per net. On the host
+// the records of 22k nets took 0.56 ms of 3.6 for loading the design, and their copy 0.1.
+__global__ void __launch_bounds__(128)
+records_kernel(const __grid_constant__ DevDesign D, uint4 *__restrict__ out) {
+    const uint32_t e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= D.n_net) return;
+    const uint32_t IR = D.I + D.R;
+    uint4 d = make_uint4(0, 0, 0, 0), ni = D.netinfo[e];
+    uint32_t c[8], l[8], end = 0;
+#pragma unroll
+    for (uint32_t k = 0; k < 8; ++k) {
+        const bool on = k < ni.y - ni.x;
+        c[k] = on ? D.fo_edge[ni.x + k] : 0u;
+        l[k] = on ? (uint32_t)(uint16_t)(D.fo_lvl[ni.x + k] << 4) : 0u;
+    }
+    if (e >= IR) {
+        d = D.desc[e - IR];
+        const uint32_t op = meta_op(d.w);
+        if (op == OP_MUX2) d = make_uint4(d.y, d.z, d.x, d.w);
+        const int no = n_operands(op);
+        d.w |= (no >= 3 ? 7u : no == 2 ? 3u : no == 1 ? 1u : 0u) << 4;
+        switch (op) {
+        case OP_AND: d.w |= PM_A; break;
+        case OP_OR: d.w |= PM_A | PM_B | PM_C; break;
+        case OP_XOR: d.w |= PM_B | PM_C; break;
+        case OP_NOT: d.w |= PM_B | PM_D; break;
+        case OP_ADD: case OP_SUB: d.w |= PM_SUM; break;
+        case OP_EQ: case OP_LT: d.w |= PM_CMP; break;
+        case OP_MUX2: d.w |= PM_C; break;
+        case OP_SHL: d.w |= PM_B | PM_LEFT; break;
+        case OP_CONCAT: d.w |= PM_B | PM_C | PM_LEFT; break;
+        case OP_SHR: case OP_SLICE: d.w |= PM_B; break;
+        default: break;
+        }
+        end = D.lvl_start[D.node_level[e - IR] + 1];
+    }
+    if (ni_nreg(ni.w) == 1) ni.z = D.dreg_rec[ni.z];
+    uint4 *const r = out + (size_t)e * 8;
+    r[0] = d;
+    r[1] = ni;
+    r[2] = make_uint4(c[0], c[1], c[2], c[3]);
+    r[3] = make_uint4(c[4], c[5], c[6], c[7]);
+    r[4] = make_uint4(l[0] | l[1] << 16, l[2] | l[3] << 16, l[4] | l[5] << 16, l[6] | l[7] << 16);
+    r[5] = make_uint4(end, 0, 0, 0);
+    r[6] = r[7] = make_uint4(0, 0, 0, 0);
+}
+
+cudaError_t launch_records(const DevDesign &d, uint4 *rec, cudaStream_t stream) {
+    if (!d.n_net) return cudaSuccess;
+    records_kernel<<<(d.n_net + 127) / 128, 128, 0, stream>>>(d, rec);
+    return cudaGetLastError();
+}
+
 // The tiers: lanes per fault, table entries per lane.
 constexpr int TIER_LPS[PACK_TIERS] = {1, 8, 32, 256}, TIER_TPL[PACK_TIERS] = {8, 16, 16, 16};
 
