@@ -292,10 +292,14 @@ static_kernel(const DevDesign *__restrict__ designs, uint32_t design, const Stat
                 }
                 __syncwarp();
             }
-            for (uint32_t i = lane; i < dt; i += 32)
-                for (uint32_t x = m.dtop[i]; x; x &= x - 1) m.df[i * 32 + __ffs((int)x) - 1] = 0u;
-            __syncwarp();
-            for (uint32_t i = lane; i < dt; i += 32) m.dtop[i] = 0u;
+            for (uint32_t i = 0; i < dt; i += 32) {   // clear df: all lanes share a word of dtop
+                const uint32_t x = i + lane < dt ? m.dtop[i + lane] : 0u;
+                for (uint32_t any = __ballot_sync(FULL, x != 0u); any; any &= any - 1) {
+                    const int src = __ffs((int)any) - 1;
+                    if (__shfl_sync(FULL, x, src) >> lane & 1u) m.df[(i + src) * 32 + lane] = 0u;
+                }
+                if (x) m.dtop[i + lane] = 0u;
+            }
             port = __reduce_min_sync(FULL, port);
             nreg = *(volatile uint32_t *)m.n_new;
             __syncwarp();
