@@ -194,7 +194,7 @@ struct rtlfs_ctx {
     cudaStream_t s_tier[PACK_TIERS - 2] = {};   // third tier on (the last with the heavy kernel)
     cudaEvent_t ev_pk[PACK_TIERS] = {};
     uint64_t w_pool_cap = 0;
-    cudaEvent_t ev_wg = nullptr, ev_wl = nullptr;
+    cudaEvent_t ev_wg = nullptr, ev_wl = nullptr, ev_upload = nullptr;
     // the good-trace launch lists of one span of cycles run side by side: the first on the
     // caller's stream, the others on these, joined back through the events
     cudaStream_t s_gaux[5] = {};
@@ -948,9 +948,11 @@ int launch_good(rtlfs_ctx *ctx, uint32_t *n_launches = nullptr) {
 
 // Host-to-device copies go through the legacy stream; one from pageable memory may return before
 // it has landed, and the context's (non-blocking) streams do not wait for that stream. Every call
-// that launches on them after such copies comes through here first.
+// that launches on them after such copies comes through here first: the main stream, behind
+// which all of a call's work starts, waits for them.
 int uploads_landed(rtlfs_ctx *ctx) {
-    CU(cudaStreamSynchronize(cudaStreamLegacy));
+    CU(cudaEventRecord(ctx->ev_upload, cudaStreamLegacy));
+    CU(cudaStreamWaitEvent(ctx->s_main, ctx->ev_upload, 0));
     return RTLFS_OK;
 }
 
@@ -1425,6 +1427,7 @@ int rtlfs_create(rtlfs_ctx **out, int device) {
         for (auto &e : ctx->ev_gjoin) CU(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
         CU(cudaEventCreateWithFlags(&ctx->ev_wg, cudaEventDisableTiming));
         CU(cudaEventCreateWithFlags(&ctx->ev_wl, cudaEventDisableTiming));
+        CU(cudaEventCreateWithFlags(&ctx->ev_upload, cudaEventDisableTiming));
         for (auto &e : ctx->ev) CU(cudaEventCreate(&e));
         for (auto &e : ctx->ev_graph) CU(cudaEventCreate(&e));
         CU(cudaEventCreate(&ctx->ev_gend));
@@ -1453,6 +1456,7 @@ void rtlfs_destroy(rtlfs_ctx *ctx) {
     for (auto &e : ctx->ev_win) if (e) cudaEventDestroy(e);
     if (ctx->ev_wg) cudaEventDestroy(ctx->ev_wg);
     if (ctx->ev_wl) cudaEventDestroy(ctx->ev_wl);
+    if (ctx->ev_upload) cudaEventDestroy(ctx->ev_upload);
     for (auto &x : ctx->s_gaux) if (x) { cudaStreamSynchronize(x); cudaStreamDestroy(x); }
     if (ctx->ev_gfork) cudaEventDestroy(ctx->ev_gfork);
     for (auto &e : ctx->ev_gjoin) if (e) cudaEventDestroy(e);
