@@ -81,8 +81,9 @@ __host__ __device__ inline size_t static_warp_bytes(uint32_t n_node, uint32_t n_
 // lanes a node each, until none is left. Which nets differ is a bitmap in shared memory, so an
 // operand is one load, of the faulty value (in the slot's part of the scratch array) or of the
 // good one. What bounds it is the chain of a level, some 1000 cycles: the search for its nodes,
-// their 128-byte records, their operands. 1500 faults of 1200 nodes over 300 cycles: 13.0 ms with a
-// thread per fault and its heap of dirty nodes in the scratch array, 4.0 so.
+// their 128-byte records, their operands. 1500 faults of 1200 nodes over 300 cycles: 11.6 ms with a
+// thread per fault and its heap of dirty nodes in the scratch array, 3.4 so. (One to four faults: 0.2 to
+// 1.6 times a thread's time; an idle fault's cycles are skipped, a busy one's level costs more.)
 // THIN: for designs with a few nodes per level, where a level's search is most of its cost. 20 and
 // 2000 faults of a 1000-level chain over 50 cycles took 56 and 64 ms without the walk (a thread per
 // fault: 44 and 49), 18 and 22 with it. Elsewhere it costs 3% (1200 nodes), so it is left out there.
